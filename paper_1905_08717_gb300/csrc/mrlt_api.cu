@@ -25,6 +25,8 @@ struct mr_solver {
     std::vector<void*> node_allocs; // node arrays of the current capacity
     double* d_part = nullptr;
     long long ntot = 0;             // cells over all levels
+    long long tpad = 0;             // entries of the tile maps, padded likewise
+    long long npad = 0;             // entries of the per-cell maps: every level padded to whole vectors
     size_t fixed_bytes = 0;         // device bytes of the fixed arrays
     int* h_top = nullptr;           // pinned: [0] free slots, [1] refinement flags of a head,
                                     // [2..3] halt record (Grid::room[1..2])
@@ -363,7 +365,7 @@ mr_status count_nodes(mr_solver* h, long long* used)
 // cell until the next macro-step boundary)
 mr_status fit_new_tree(mr_solver* h)
 {
-    MR_CK(cudaMemsetAsync(h->K.g.flag, 0, (size_t)h->ntot, h->stream)); // (see adapt)
+    MR_CK(cudaMemsetAsync(h->K.g.flag, 0, (size_t)h->npad, h->stream)); // (see adapt)
     long long used = 0;
     MR_TRY(count_nodes(h, &used));
     h->used_macro = used;
@@ -948,7 +950,9 @@ mr_status init_state(mr_solver* h, const double* q0)
     const size_t esz = g.prec ? sizeof(float) : sizeof(double); // field element
     for (int f = 0; f < NFIELD; ++f) MR_CK(cudaMemsetAsync(g.f[f], 0, (size_t)g.cap * m * esz, h->stream));
     if (g.rg) MR_CK(cudaMemsetAsync(g.rg, 0, (size_t)g.cap * g.nf * m * sizeof(double), h->stream));
-    MR_CK(cudaMemsetAsync(g.flag, 0, h->ntot, h->stream));
+    MR_CK(cudaMemsetAsync(g.flag, 0, h->npad, h->stream));
+    MR_CK(cudaMemsetAsync(g.st, 0, h->npad, h->stream)); // the padding holds no node
+    MR_CK(cudaMemsetAsync(g.tflag, 0, h->tpad, h->stream));
     MR_CK(cudaMemsetAsync(g.counts, 0, 3 * (LMAX + 1) * sizeof(int), h->stream));
     MR_CK(cudaMemsetAsync(g.err, 0, sizeof(int), h->stream));
     MR_CK(cudaMemsetAsync(g.room, 0, 4 * sizeof(int), h->stream));
@@ -1004,6 +1008,8 @@ mr_status layout_alloc(mr_solver* h, const mr_config* cfg)
     g.igm = cfg->equation == MR_EQ_EULER ? 1.0 / (cfg->phys[0] - 1.0) : 0.0;
     g.gcap = 0;
     long long off = 0, toff = 0;
+    h->ntot = 0;
+    auto pad16 = [](long long n) { return (n + 15) / 16 * 16; }; // 16-byte vectors of the byte maps
     for (int l = g.lb; l <= g.L; ++l) {
         g.toff[l] = toff;
         const long long nl = 1LL << l;
@@ -1012,19 +1018,20 @@ mr_status layout_alloc(mr_solver* h, const mr_config* cfg)
         g.ntx[l] = (int)((nl + tx - 1) / tx);
         g.nty[l] = g.d >= 2 ? (int)((nl + ty - 1) / ty) : 1;
         g.ntz[l] = g.d == 3 ? (int)((nl + kTile3Z - 1) / kTile3Z) : 1;
-        toff += (long long)g.ntx[l] * g.nty[l] * g.ntz[l];
+        toff += pad16((long long)g.ntx[l] * g.nty[l] * g.ntz[l]);
         g.off[l] = off;
         g.N[l] = 1LL << (g.d * l);
+        h->ntot += g.N[l];
         g.n[l] = 1 << l;
         for (int k = 0; k < 3; ++k) {
             g.dx[l][k] = (cfg->hi[k] - cfg->lo[k]) / g.n[l];
             g.rdx[l][k] = 1.0 / g.dx[l][k];
         }
-        off += g.N[l];
+        off += pad16(g.N[l]);
     }
-    h->ntot = off;
+    h->npad = off;
+    h->tpad = toff;
     h->reg = cfg->reflux && !g.gts;
-    const size_t nd = (size_t)off * g.m;
     mr_status r = MR_OK;
     auto A = [&](mr_status s) {
         if (r == MR_OK) r = s;
@@ -1051,19 +1058,17 @@ mr_status layout_alloc(mr_solver* h, const mr_config* cfg)
     if (r == MR_OK && !h->dry &&
         cudaMemsetAsync(g.work, 0, (LMAX + 1) * 4 * sizeof(unsigned long long), h->stream) != cudaSuccess)
         r = MR_E_CUDA; // cumulative counters: never cleared by mr_reset
-    long long nblk = 0;
-    for (int l = g.lb; l <= g.L; ++l) nblk += (g.N[l] + NTHREADS - 1) / NTHREADS;
-    A(dev_alloc(h, &h->K.bc, 2 * nblk));
+    LevelChunks lc;
+    A(dev_alloc(h, &h->K.bc, 2 * (size_t)number_chunks(g, lc, g.lb, g.L)));
     A(dev_alloc(h, &h->d_part, (size_t)(LMAX + 1) * MASS_BLOCKS * g.m));
-    (void)nd;
     h->fixed_bytes = h->bytes;
     // node arrays: the full tree of a new solver (every cell a node) plus the sink
     if (h->dry) {
-        h->bytes += (size_t)(off + 1) * per_node_bytes(g, h->reg);
-        g.cap = off + 1;
+        h->bytes += (size_t)(h->ntot + 1) * per_node_bytes(g, h->reg);
+        g.cap = h->ntot + 1;
     } else if (r == MR_OK) {
-        r = alloc_nodes(h, g, off + 1, h->node_allocs);
-        h->bytes = h->fixed_bytes + (size_t)(off + 1) * per_node_bytes(g, h->reg);
+        r = alloc_nodes(h, g, h->ntot + 1, h->node_allocs);
+        h->bytes = h->fixed_bytes + (size_t)(h->ntot + 1) * per_node_bytes(g, h->reg);
     }
     if (r == MR_OK && !h->dry && !h->h_top) {
         if (cudaMallocHost((void**)&h->h_top, 4 * sizeof(int)) != cudaSuccess) {
@@ -1192,8 +1197,8 @@ mr_status mr_set_tree(mr_solver* h, const unsigned char* lev)
         }
     h->K.leaf_copy(lb, L, F_QE, F_Q0);
     for (int l = L - 1; l >= lb; --l) h->K.project(l, PM_Q0);
-    MR_CK(cudaMemsetAsync(g.flag, 0, h->ntot, h->stream));
-    std::vector<uint8_t> fl((size_t)h->ntot, 0);
+    MR_CK(cudaMemsetAsync(g.flag, 0, h->npad, h->stream));
+    std::vector<uint8_t> fl((size_t)h->npad, 0);
     for (int l = lb; l < L; ++l)
         for (long long id = 0; id < g.N[l]; ++id)
             if (R[l][id]) fl[g.off[l] + id] = FL_REF;
@@ -1488,8 +1493,8 @@ mr_status mr_read(mr_solver* h, int what, void* buf, size_t cap, size_t* used)
     } else if (what == MR_READ_UNIFORM) { // a transient pyramid for the inverse transform
         double* T = nullptr;
         uint8_t* us = nullptr;
-        MR_TRY(scratch(h, &T, (size_t)h->ntot * m));
-        MR_TRY(scratch(h, &us, (size_t)h->ntot));
+        MR_TRY(scratch(h, &T, (size_t)h->npad * m));
+        MR_TRY(scratch(h, &us, (size_t)h->npad));
         h->K.uniform(T, us);
         MR_CK(cudaMemcpyAsync(buf, T + g.off[g.L] * m, need, cudaMemcpyDeviceToHost, h->stream));
         MR_CK(cudaFreeAsync(T, h->stream));

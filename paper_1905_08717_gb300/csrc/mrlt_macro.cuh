@@ -231,31 +231,15 @@ k_macro(const __grid_constant__ Grid g, MacroArgs a)
                 mph_apply<D, M, R>(g, l, la);
                 MRLT_SYNC();
             }
-            // leaf, node and active-tile lists of levels la..L (chunks of NT cells)
+            // leaf, node and active-tile lists of levels la..L
             LevelChunks lc;
-            lc.lo = la;
-            lc.hi = L;
-            int total = 0;
-            for (int l = la; l <= L; ++l) {
-                lc.base[l] = total;
-                total += (int)((g.N[l] + NT - 1) / NT);
-            }
-            lc.base[L + 1] = total;
+            const int total = number_chunks(g, lc, la, L);
             phase(PH_ADAPT, 6);
-            {
-                const long long t0 = g.toff[la], t1 = g.toff[L] + (long long)g.ntx[L] * g.nty[L] * g.ntz[L];
-                MRLT_GRID_STRIDE(i, t1 - t0) g.tflag[t0 + i] = 0;
-            }
             for (int c = blockIdx.x; c < total; c += gridDim.x) chunk_count<NT>(g, lc, c, a.bc);
             MRLT_SYNC();
             phase(PH_ADAPT, 7);
-            for (int l = la + blockIdx.x; l <= L; l += gridDim.x) level_scan<NT>(g, lc, l, a.bc);
-            MRLT_SYNC();
-            phase(PH_ADAPT, 8);
+            for (int l = L - blockIdx.x; l >= la; l -= gridDim.x) level_tile_list<NT>(g, l);
             for (int c = blockIdx.x; c < total; c += gridDim.x) chunk_scatter<NT>(g, lc, c, a.bc);
-            MRLT_SYNC();
-            phase(PH_ADAPT, 9);
-            for (int l = la + blockIdx.x; l <= L; l += gridDim.x) level_tile_list<NT>(g, l);
             MRLT_SYNC();
             for (int l = L - 1; l >= la; --l) {
                 phase(PH_ADAPT, 10);

@@ -95,33 +95,20 @@ __global__ void k_release_apply(const __grid_constant__ Grid g, int la)
     dev_apply<D, M, T>(g, la, la);
 }
 
-// compaction of levels lo..hi: chunks of NTHREADS cells, one block each;
-// the tile flags of those levels [t0, t1) cleared for the scatter
-__global__ void k_cmp_count(const __grid_constant__ Grid g, LevelChunks lc, int* bc, long long t0, long long t1)
+// compaction of levels lo..hi: one block per chunk
+__global__ void k_cmp_count(const __grid_constant__ Grid g, LevelChunks lc, int* bc)
 {
     MRLT_ENTER(g);
     chunk_count<NTHREADS>(g, lc, blockIdx.x, bc);
-    MRLT_GRID_STRIDE(i, t1 - t0) g.tflag[t0 + i] = 0;
 }
 
-// exclusive scan of the per-chunk counts, one block per level
-__global__ void k_cmp_scan(const __grid_constant__ Grid g, LevelChunks lc, int* bc)
-{
-    MRLT_ENTER(g);
-    level_scan<1024>(g, lc, lc.lo + blockIdx.x, bc);
-}
-
+// the tile lists (the longest single blocks) first, then one block per chunk
 __global__ void k_cmp_scatter(const __grid_constant__ Grid g, LevelChunks lc, const int* bc)
 {
     MRLT_ENTER(g);
-    chunk_scatter<NTHREADS>(g, lc, blockIdx.x, bc);
-}
-
-// ordered list of the active tiles of level lo + blockIdx.x (one block per level)
-__global__ void k_tile_list(const __grid_constant__ Grid g, int lo)
-{
-    MRLT_ENTER(g);
-    level_tile_list<1024>(g, lo + blockIdx.x);
+    const int levels = lc.hi - lc.lo + 1;
+    if ((int)blockIdx.x < levels) level_tile_list<NTHREADS>(g, lc.hi - blockIdx.x);
+    else chunk_scatter<NTHREADS>(g, lc, blockIdx.x - levels, bc);
 }
 
 template <int D, class T>
@@ -368,21 +355,11 @@ void Launcher::apply_tree(int la) { MRLT_DM_DISPATCH(apply_dm, *this, la); }
 
 void Launcher::compact(int lo, int hi)
 {
-    LevelChunks lbk;
-    lbk.lo = lo;
-    lbk.hi = hi;
-    int total = 0;
-    for (int l = lo; l <= hi; ++l) {
-        lbk.base[l] = total;
-        total += (int)((g.N[l] + NTHREADS - 1) / NTHREADS);
-    }
-    lbk.base[hi + 1] = total;
-    const long long t0 = g.toff[lo], t1 = g.toff[hi] + (long long)g.ntx[hi] * g.nty[hi] * g.ntz[hi];
-    pdl_launch(k_cmp_count, total, NTHREADS, 0, st, g, lbk, bc, t0, t1);
-    pdl_launch(k_cmp_scan, hi - lo + 1, 1024, 0, st, g, lbk, bc);
-    pdl_launch(k_cmp_scatter, total, NTHREADS, 0, st, g, lbk, (const int*)bc);
-    pdl_launch(k_tile_list, hi - lo + 1, 1024, 0, st, g, lo);
-    n += 4;
+    LevelChunks lc;
+    const int total = number_chunks(g, lc, lo, hi);
+    pdl_launch(k_cmp_count, total, NTHREADS, 0, st, g, lc, bc);
+    pdl_launch(k_cmp_scatter, total + hi - lo + 1, NTHREADS, 0, st, g, lc, (const int*)bc);
+    n += 2;
 }
 
 template <class T>
@@ -468,12 +445,16 @@ void Launcher::store_finest(const double* src)
     ++n;
 }
 
-// every cell of levels lb..L a node in slot 1 + (its offset in the
-// pyramid): the full tree of a new solver; the free stack holds the rest
+// every cell of levels lb..L a node, in level and cell order from slot 1 on:
+// the full tree of a new solver; the free stack holds the rest
 __global__ void k_slots_full(Grid g, long long ntot)
 {
     pdl_enter();
-    GRID_STRIDE(i, ntot) g.slot[g.off[g.lb] + i] = (int)(1 + i);
+    long long first = 1;
+    for (int l = g.lb; l <= g.L; ++l) {
+        GRID_STRIDE(i, g.N[l]) g.slot[g.off[l] + i] = (int)(first + i);
+        first += g.N[l];
+    }
     const long long nfree = g.cap - 1 - ntot;
     GRID_STRIDE(k, nfree) g.fstack[k] = (int)(g.cap - 1 - k);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
