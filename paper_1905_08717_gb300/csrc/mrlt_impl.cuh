@@ -48,7 +48,7 @@ constexpr int kTileThreads1 = 128, kTileThreads2 = 256, kTileThreads3 = 256;
 
 enum Field { F_Q0 = 0, F_Q1, F_Q2, F_QE, F_XH, F_NH, F_N1, F_N3, NFIELD };
 enum Kind { K_WALL = 0, K_LEAF = 1, K_FINER = 2, K_COARSER = 3 };
-enum FlagBits { FL_SIG = 1, FL_BIG = 2, FL_DES = 4, FL_ALLOW = 8, FL_REF = 16 };
+enum FlagBits { FL_SIG = 1, FL_BIG = 2, FL_REF = 16 };
 enum ErrBits { ERR_INDEX = 1, ERR_SOURCE = 2, ERR_NONFINITE = 4, ERR_REFLUX = 8, ERR_TIMEOUT = 16, ERR_CAPACITY = 32 };
 
 struct Grid {

@@ -130,14 +130,9 @@ __device__ __noinline__ void mph_detail(const Grid& g, int lo, int hi)
     dev_detail<D, M, T>(g, lo, hi);
 }
 template <int D>
-__device__ __noinline__ void mph_desire(const Grid& g, int lo, int hi, int la)
+__device__ __noinline__ void mph_mark(const Grid& g, int lo, int hi, int la)
 {
-    dev_desire<D>(g, lo, hi, la);
-}
-template <int D>
-__device__ __noinline__ void mph_allow(const Grid& g, int lo, int hi, int la)
-{
-    dev_allow<D>(g, lo, hi, la);
+    dev_mark<D>(g, lo, hi, la);
 }
 template <int D>
 __device__ __noinline__ void mph_close(const Grid& g, int l)
@@ -147,7 +142,7 @@ __device__ __noinline__ void mph_close(const Grid& g, int l)
 template <int D, int M, class T>
 __device__ __noinline__ void mph_apply(const Grid& g, int l, int la)
 {
-    dev_apply<D, M, T>(g, l, la);
+    dev_apply<D, M, T, Tile<D>::THREADS>(g, l, la);
 }
 template <int D, class T>
 __device__ __noinline__ void mph_reflux(const Grid& g, int lo, int hi)
@@ -213,10 +208,7 @@ k_macro(const __grid_constant__ Grid g, MacroArgs a)
             mph_detail<D, M, R>(g, la, L - 1);
             MRLT_SYNC();
             phase(PH_ADAPT, 2);
-            mph_desire<D>(g, la, L - 1, la);
-            MRLT_SYNC();
-            phase(PH_ADAPT, 3);
-            mph_allow<D>(g, la, L - 1, la);
+            mph_mark<D>(g, la, L - 1, la);
             MRLT_SYNC();
             for (int l = L - 1; l > la; --l) {
                 phase(PH_ADAPT, 4);

@@ -12,6 +12,11 @@ static inline int blocks_dense(long long n)
     long long b = (n + NTHREADS - 1) / NTHREADS;
     return (int)(b < 1 ? 1 : (b > 65535 ? 65535 : b));
 }
+// blocks of the passes that take 16 cells per thread
+static inline int blocks_step(const Grid& g, int l)
+{
+    return blocks_dense(l < kStepLevel ? g.N[l] : g.N[l] / kStep);
+}
 static inline int blocks_list(const Grid& g, int l)
 {
     long long b = (g.N[l] + NTHREADS - 1) / NTHREADS;
@@ -53,17 +58,15 @@ __global__ void k_detail(const __grid_constant__ Grid g, int lo, int hi)
     dev_detail<D, M, T>(g, lo, hi);
 }
 
-// Desired and admissible refinements in one pass: a cell's admissibility
-// reads only its own desire bit (set by the same thread, same grid-stride
-// order), and desire reads only the detail bits, which admissibility keeps.
+// Desired and admissible refinements in one pass: desire reads only the detail
+// bits, which the stores of the refinement bit keep.
 // it >= 0: this launch finalises the refinement flags (a remesh at level
 // la = L-1 has no closure), so it also checks that the new tree fits.
 template <int D>
 __global__ void k_mark(const __grid_constant__ Grid g, int lo, int hi, int la, long long it)
 {
     MRLT_ENTER(g);
-    dev_desire<D>(g, lo, hi, la);
-    dev_allow<D>(g, lo, hi, la);
+    dev_mark<D>(g, lo, hi, la);
     if (it >= 0) room_decide(g, refined_here(g, la), la, it);
 }
 
@@ -81,7 +84,7 @@ template <int D, int M, class T>
 __global__ void k_apply(const __grid_constant__ Grid g, int l, int la)
 {
     MRLT_ENTER(g);
-    dev_apply<D, M, T>(g, l, la);
+    dev_apply<D, M, T, NTHREADS>(g, l, la);
 }
 
 // the releases of a remesh and its installation on level la in one launch:
@@ -92,7 +95,7 @@ __global__ void k_release_apply(const __grid_constant__ Grid g, int la)
 {
     MRLT_ENTER(g);
     dev_release(g, la);
-    dev_apply<D, M, T>(g, la, la);
+    dev_apply<D, M, T, NTHREADS>(g, la, la);
 }
 
 // compaction of levels lo..hi: one block per chunk
@@ -319,10 +322,10 @@ static void adapt_dm(Launcher& L, int la, long long it)
     const int hi = g.L - 1; // levels whose nodes may own children
     if (g.prec) pdl_launch(k_detail<D, M, float>, blocks_list(g, hi), NTHREADS, 0, L.st, g, la, hi);
     else pdl_launch(k_detail<D, M, double>, blocks_list(g, hi), NTHREADS, 0, L.st, g, la, hi);
-    pdl_launch(k_mark<D>, blocks_dense(g.N[hi]), NTHREADS, 0, L.st, g, la, hi, la, la == hi ? it : -1LL);
+    pdl_launch(k_mark<D>, blocks_step(g, hi), NTHREADS, 0, L.st, g, la, hi, la, la == hi ? it : -1LL);
     L.n += 2;
     for (int l = g.L - 1; l > la; --l, ++L.n)
-        pdl_launch(k_close<D>, blocks_dense(g.N[l - 1]), NTHREADS, 0, L.st, g, l, l == la + 1 ? it : -1LL);
+        pdl_launch(k_close<D>, blocks_step(g, l - 1), NTHREADS, 0, L.st, g, l, l == la + 1 ? it : -1LL);
 }
 
 
@@ -330,13 +333,13 @@ template <int D, int M>
 static void apply_dm(Launcher& L, int la)
 {
     const Grid& g = L.g;
-    const int b0 = blocks_list(g, g.L), b1 = blocks_dense(g.N[la]);
+    const int b0 = blocks_list(g, g.L), b1 = blocks_step(g, la);
     if (g.prec) pdl_launch(k_release_apply<D, M, float>, b0 > b1 ? b0 : b1, NTHREADS, 0, L.st, g, la);
     else pdl_launch(k_release_apply<D, M, double>, b0 > b1 ? b0 : b1, NTHREADS, 0, L.st, g, la);
     ++L.n;
     for (int l = la + 1; l <= g.L; ++l, ++L.n) {
-        if (g.prec) pdl_launch(k_apply<D, M, float>, blocks_dense(g.N[l]), NTHREADS, 0, L.st, g, l, la);
-        else pdl_launch(k_apply<D, M, double>, blocks_dense(g.N[l]), NTHREADS, 0, L.st, g, l, la);
+        if (g.prec) pdl_launch(k_apply<D, M, float>, blocks_step(g, l), NTHREADS, 0, L.st, g, l, la);
+        else pdl_launch(k_apply<D, M, double>, blocks_step(g, l), NTHREADS, 0, L.st, g, l, la);
     }
 }
 
