@@ -551,7 +551,7 @@ mr_status adapt(mr_solver* h, int la, int part = 0, long long it = 0)
     if (part != 2) {
         if (la == g.lb) {
             h->K.scale_init();
-            for (int l = g.lb; l <= g.L; ++l) h->K.scale(l);
+            h->K.scale();
         }
         // the flags are zero here: every remesh's compaction clears those it set
         h->K.mark_refinements(la, part == 0 && can_halt(h) ? it : -1);
@@ -623,7 +623,7 @@ mr_status gts_iteration(mr_solver* h, long long n, int part = 0)
 
 mr_status finite_check(mr_solver* h)
 {
-    for (int l = h->K.g.lb; l <= h->K.g.L; ++l) h->K.finite(l);
+    h->K.finite();
     if (h->async_err) {
         MR_CK(cudaMemcpyAsync(h->async_err, h->K.g.err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
         return MR_OK;
@@ -907,10 +907,8 @@ mr_status cfl_enqueue(mr_solver* h, unsigned long long* bits)
         return MR_OK;
     }
     MR_CK(cudaMemsetAsync(g.wmax, 0, sizeof(unsigned long long), h->stream));
-    for (int l = g.lb; l <= g.L; ++l) {
-        launch_wave(g, h->stream, l);
-        ++h->stage_launches;
-    }
+    launch_wave(g, h->stream);
+    ++h->stage_launches;
     MR_CK(cudaMemcpyAsync(bits, g.wmax, sizeof *bits, cudaMemcpyDeviceToHost, h->stream));
     return MR_OK;
 }
@@ -1467,11 +1465,7 @@ mr_status mr_read(mr_solver* h, int what, void* buf, size_t cap, size_t* used)
         MR_TRY(scratch(h, &tmp, need));
         int* keys = what == MR_READ_LEAF_KEYS ? (int*)tmp : nullptr;
         double* vals = what == MR_READ_LEAF_VALUES ? (double*)tmp : nullptr;
-        long long base = 0;
-        for (int l = g.lb; l <= g.L; ++l) {
-            if (cnt[l]) h->K.pack(l, base, keys, vals);
-            base += cnt[l];
-        }
+        h->K.pack(keys, vals);
         if (need) MR_CK(cudaMemcpyAsync(buf, tmp, need, cudaMemcpyDeviceToHost, h->stream));
         MR_CK(cudaFreeAsync(tmp, h->stream));
     } else if (what == MR_READ_PROFILE) {

@@ -31,6 +31,7 @@
 //   pops until the next compaction commits them).
 #pragma once
 #include <cstdint>
+#include <cstring>
 #include <cuda_runtime.h>
 
 namespace mrlt {
@@ -633,7 +634,7 @@ struct Launch; // fwd
 // mode), RK weight b of the stage; returns the number of kernel launches issued
 // (-1 when the kernel could not be set up).  lo > hi only sets the kernel up.
 int launch_stage(const Grid& g, cudaStream_t st, int lo, int hi, int s, int lmin, double b, int reg);
-void launch_wave(const Grid& g, cudaStream_t st, int l);
+void launch_wave(const Grid& g, cudaStream_t st);
 // one persistent macro-step kernel launch (mrlt_macro.cuh); a == nullptr sets
 // the kernel up only.  Returns 1 when launched, 0 after set-up, -1 on failure.
 struct MacroArgs;

@@ -119,10 +119,10 @@ __device__ __noinline__ void mph_stage(const Grid& g, int lo, int hi, int s, int
 {
     stage_tiles<EQ, D, R>(g, lo, hi, s, lmin, b, reg, smem);
 }
-template <int D, class T>
+template <int D, int M, class T>
 __device__ __noinline__ void mph_project(const Grid& g, int l, int mode)
 {
-    dev_project<D, T>(g, l, mode);
+    dev_project<D, M, T>(g, l, mode);
 }
 template <int D, int M, class T>
 __device__ __noinline__ void mph_detail(const Grid& g, int lo, int hi)
@@ -144,15 +144,15 @@ __device__ __noinline__ void mph_apply(const Grid& g, int l, int la)
 {
     dev_apply<D, M, T, Tile<D>::THREADS>(g, l, la);
 }
-template <int D, class T>
+template <int D, int M, class T>
 __device__ __noinline__ void mph_reflux(const Grid& g, int lo, int hi)
 {
-    dev_reflux<D, T>(g, lo, hi);
+    dev_reflux<D, M, T>(g, lo, hi);
 }
 template <int EQ, int D, class T>
 __device__ __noinline__ void mph_end(const Grid& g, int lo, int hi)
 {
-    dev_finite<T>(g, lo, hi);
+    dev_finite<EQ == 2 ? D + 2 : 1, T>(g, lo, hi);
     dev_wave<EQ, D, T>(g, lo, hi);
 }
 
@@ -191,17 +191,17 @@ k_macro(const __grid_constant__ Grid g, MacroArgs a)
         phase(PH_TREE, L);
         if (adapt_now && lmin == lb && lead)
             for (int v = 0; v < MMAX; ++v) g.scale_bits[v] = (unsigned long long)__double_as_longlong(1e-14);
-        dev_leaf_copy<R>(g, lmin, L, F_QE, F_Q0);
+        dev_leaf_copy<M, R>(g, lmin, L, F_QE, F_Q0);
         MRLT_SYNC();
         for (int l = L - 1; l >= lmin; --l) {
             phase(PH_TREE, l);
-            mph_project<D, R>(g, l, PM_Q0);
+            mph_project<D, M, R>(g, l, PM_Q0);
             MRLT_SYNC();
         }
         if (adapt_now) { // restricted remesh of levels >= la = lmin (Sec. 4)
             const int la = lmin;
             phase(PH_ADAPT, 0);
-            if (la == lb) dev_scale<R>(g, lb, L);
+            if (la == lb) dev_scale<M, R>(g, lb, L);
             dev_clear_flags(g, g.off[la], g.off[L] + g.N[L]);
             MRLT_SYNC();
             phase(PH_ADAPT, 1);
@@ -235,7 +235,7 @@ k_macro(const __grid_constant__ Grid g, MacroArgs a)
             MRLT_SYNC();
             for (int l = L - 1; l >= la; --l) {
                 phase(PH_ADAPT, 10);
-                mph_project<D, R>(g, l, PM_Q0);
+                mph_project<D, M, R>(g, l, PM_Q0);
                 MRLT_SYNC();
             }
         }
@@ -244,7 +244,7 @@ k_macro(const __grid_constant__ Grid g, MacroArgs a)
                 if (s > 1)
                     for (int l = L - 1; l >= lb; --l) {
                         phase(PH_TREE, l);
-                        mph_project<D, R>(g, l, s == 2 ? PM_Q1 : PM_Q2);
+                        mph_project<D, M, R>(g, l, s == 2 ? PM_Q1 : PM_Q2);
                         MRLT_SYNC();
                     }
                 phase(PH_STAGE1 + s - 1, L);
@@ -255,7 +255,7 @@ k_macro(const __grid_constant__ Grid g, MacroArgs a)
         }
         if (lmin > lb) { // Alg. 3 / Sec. 4.3: the mid-step level lmin - 1
             phase(PH_TREE, lmin - 1);
-            mph_project<D, R>(g, lmin - 1, PM_MID);
+            mph_project<D, M, R>(g, lmin - 1, PM_MID);
             MRLT_SYNC();
         }
         // first RK stage on every active level (independent levels: one phase)
@@ -264,13 +264,13 @@ k_macro(const __grid_constant__ Grid g, MacroArgs a)
         MRLT_SYNC();
         for (int l = L - 1; l >= lmin; --l) { // Alg. 8
             phase(PH_TREE, l);
-            mph_project<D, R>(g, l, PM_REF2);
+            mph_project<D, M, R>(g, l, PM_REF2);
             MRLT_SYNC();
         }
         for (int l = L; l >= lmin; --l) { // Alg. 5 with the Alg. 4 projections
             if (l < L) {
                 phase(PH_TREE, l);
-                mph_project<D, R>(g, l, PM_PRJ2);
+                mph_project<D, M, R>(g, l, PM_PRJ2);
                 MRLT_SYNC();
             }
             phase(PH_STAGE2, l);
@@ -280,13 +280,13 @@ k_macro(const __grid_constant__ Grid g, MacroArgs a)
         if (g.rk == 3) {
             for (int l = L - 1; l >= lmin; --l) { // Alg. 9
                 phase(PH_TREE, l);
-                mph_project<D, R>(g, l, PM_REF3);
+                mph_project<D, M, R>(g, l, PM_REF3);
                 MRLT_SYNC();
             }
             for (int l = L; l >= lmin; --l) { // Alg. 7 with the Alg. 6 projections
                 if (l < L) {
                     phase(PH_TREE, l);
-                    mph_project<D, R>(g, l, PM_PRJ3);
+                    mph_project<D, M, R>(g, l, PM_PRJ3);
                     MRLT_SYNC();
                 }
                 phase(PH_STAGE3, l);
@@ -298,7 +298,7 @@ k_macro(const __grid_constant__ Grid g, MacroArgs a)
             const int lc = (n + 1 == a.nit) ? lb : level_min_dev(g, n + 1);
             if (lc < L) {
                 phase(PH_TREE, lc);
-                mph_reflux<D, R>(g, lc, L - 1);
+                mph_reflux<D, M, R>(g, lc, L - 1);
                 MRLT_SYNC();
             }
         }

@@ -5,12 +5,12 @@
 
 namespace mrlt {
 
-// largest sum of characteristic speeds over the leaves of level l (CFL step)
+// largest sum of characteristic speeds over all leaves (CFL step)
 template <int EQ, int D, class T>
-__global__ void __launch_bounds__(NTHREADS) k_wave(const __grid_constant__ Grid g, int l)
+__global__ void __launch_bounds__(NTHREADS) k_wave(const __grid_constant__ Grid g)
 {
     pdl_enter();
-    dev_wave<EQ, D, T>(g, l, l);
+    dev_wave<EQ, D, T>(g, g.lb, g.L);
 }
 
 int launch_stage(const Grid& g, cudaStream_t st, int lo, int hi, int s, int lmin, double b, int reg)
@@ -51,12 +51,12 @@ int launch_grid_wait_test(cudaStream_t st, int ctas, int missing, unsigned long 
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-void launch_wave(const Grid& g, cudaStream_t st, int l)
+void launch_wave(const Grid& g, cudaStream_t st)
 {
 #define MRLT_CASE(E, DD)                                                                         \
     if (g.eq == E && g.d == DD) {                                                                \
-        if (g.prec) k_wave<E, DD, float><<<grid_for(g, l), NTHREADS, 0, st>>>(g, l);            \
-        else k_wave<E, DD, double><<<grid_for(g, l), NTHREADS, 0, st>>>(g, l);                  \
+        if (g.prec) k_wave<E, DD, float><<<grid_for(g, g.L), NTHREADS, 0, st>>>(g);            \
+        else k_wave<E, DD, double><<<grid_for(g, g.L), NTHREADS, 0, st>>>(g);                  \
         return;                                                                                  \
     }
     MRLT_CASE(0, 1) MRLT_CASE(0, 2) MRLT_CASE(0, 3)

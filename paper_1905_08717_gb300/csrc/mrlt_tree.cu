@@ -29,26 +29,26 @@ static inline int blocks_list(const Grid& g, int l)
 // Each kernel waits for its predecessor (programmatic dependent launch) and
 // runs one device body of mrlt_tree_dev.cuh over its own grid.
 // (T: the storage type of the fields, double or float)
-template <class T>
+template <int M, class T>
 __global__ void k_leaf_copy(const __grid_constant__ Grid g, int lo, int hi, int from, int to)
 {
     MRLT_ENTER(g);
-    dev_leaf_copy<T>(g, lo, hi, from, to);
+    dev_leaf_copy<M, T>(g, lo, hi, from, to);
 }
 
-template <int D, class T>
+template <int D, int M, class T>
 __global__ void k_project(const __grid_constant__ Grid g, int l, int mode)
 {
     MRLT_ENTER(g);
-    dev_project<D, T>(g, l, mode);
+    dev_project<D, M, T>(g, l, mode);
 }
 
 // up-sweep of levels hi..lo in one launch (dev_project_up)
-template <int D, class T>
+template <int D, int M, class T>
 __global__ void k_project_up(const __grid_constant__ Grid g, int hi, int lo, int mode)
 {
     MRLT_ENTER(g);
-    dev_project_up<D, T>(g, hi, lo, mode);
+    dev_project_up<D, M, T>(g, hi, lo, mode);
 }
 
 template <int D, int M, class T>
@@ -114,26 +114,26 @@ __global__ void k_cmp_scatter(const __grid_constant__ Grid g, LevelChunks lc, co
     else chunk_scatter<NTHREADS>(g, lc, blockIdx.x - levels, bc);
 }
 
-template <int D, class T>
+template <int D, int M, class T>
 __global__ void k_reflux(const __grid_constant__ Grid g, int lo, int hi)
 {
     MRLT_ENTER(g);
-    dev_reflux<D, T>(g, lo, hi);
+    dev_reflux<D, M, T>(g, lo, hi);
 }
 
 // ------------------------------------------------------------ reductions
-template <class T>
-__global__ void k_scale(const __grid_constant__ Grid g, int l)
+template <int M, class T>
+__global__ void k_scale(const __grid_constant__ Grid g)
 {
     MRLT_ENTER(g);
-    dev_scale<T>(g, l, l);
+    dev_scale<M, T>(g, g.lb, g.L);
 }
 
-template <class T>
-__global__ void k_finite(const __grid_constant__ Grid g, int l)
+template <int M, class T>
+__global__ void k_finite(const __grid_constant__ Grid g)
 {
     MRLT_ENTER(g);
-    dev_finite<T>(g, l, l);
+    dev_finite<M, T>(g, g.lb, g.L);
 }
 
 // fixed-shape partial sums (deterministic): part[block * m + v]
@@ -163,29 +163,25 @@ __global__ void k_mass(Grid g, int l, double* part)
     }
 }
 
-template <class T>
-__global__ void k_pack(Grid g, int l, long long base, int* keys, double* vals)
+template <int M, class T>
+__global__ void k_pack(const __grid_constant__ Grid g, int* keys, double* vals)
 {
     pdl_enter();
-    const int cnt = g.counts[l];
-    const int* list = g.leaves + g.off[l];
-    const long long N = g.N[l];
-    GRID_STRIDE(t, cnt)
-    {
-        const long long id = list[t];
-        if (id < 0 || id >= N) continue;
-        int c[3];
-        cell_xyz(g, l, id, c);
+    for_list<0>(g, g.lb, g.L, [&](int l, long long id, long long t) {
         if (keys) {
-            int* K = keys + (base + t) * 4;
-            K[0] = l;
-            K[1] = c[0];
-            K[2] = c[1];
-            K[3] = c[2];
+            int c[3];
+            cell_xyz(g, l, id, c);
+            reinterpret_cast<int4*>(keys)[t] = make_int4(l, c[0], c[1], c[2]);
         }
-        if (vals)
-            for (int v = 0; v < g.m; ++v) vals[(base + t) * g.m + v] = double(nd<T>(g, F_QE, slot_of(g, l, id))[v]);
-    }
+        if (vals) {
+            T q[M];
+            load_row<M, T>(nd<T>(g, F_QE, slot_of(g, l, id)), q);
+            double r[M];
+#pragma unroll
+            for (int v = 0; v < M; ++v) r[v] = double(q[v]);
+            store_row<M, double>(vals + t * M, r);
+        }
+    });
 }
 
 // inverse MR transform onto the finest level, in scratch pyramids T / us:
@@ -251,69 +247,70 @@ __global__ void k_uni_down(Grid g, int l, double* T, uint8_t* us)
 }
 
 // ------------------------------------------------------------ launchers
-template <int D, class T>
-static void project_d(Launcher& L, int l, int mode)
-{
-    pdl_launch(k_project<D, T>, blocks_list(L.g, l), NTHREADS, 0, L.st, L.g, l, mode);
-}
-
-// a kernel template of the fields' storage type: float in the mixed mode
-#define MRLT_T_DISPATCH(fn, ...)              \
-    do {                                      \
-        if (g.prec) fn<float>(__VA_ARGS__);   \
-        else fn<double>(__VA_ARGS__);         \
+// fn<D, M>(...) for the solver's dimension and number of variables
+#define MRLT_DM_DISPATCH(fn, ...)                                   \
+    do {                                                            \
+        if (g.d == 1 && g.m == 1) fn<1, 1>(__VA_ARGS__);            \
+        else if (g.d == 1) fn<1, 3>(__VA_ARGS__);                   \
+        else if (g.d == 2 && g.m == 1) fn<2, 1>(__VA_ARGS__);       \
+        else if (g.d == 2) fn<2, 4>(__VA_ARGS__);                   \
+        else if (g.m == 1) fn<3, 1>(__VA_ARGS__);                   \
+        else fn<3, 5>(__VA_ARGS__);                                 \
     } while (0)
 
-void Launcher::project(int l, int mode)
+// launch k<..., T> with the fields' storage type: float in the mixed mode
+#define MRLT_T_LAUNCH(L, blocks, args, ...)                                                                    \
+    do {                                                                                                       \
+        if ((L).g.prec) pdl_launch(__VA_ARGS__, float>, blocks, NTHREADS, 0, (L).st, MRLT_UNPACK args);        \
+        else pdl_launch(__VA_ARGS__, double>, blocks, NTHREADS, 0, (L).st, MRLT_UNPACK args);                  \
+    } while (0)
+#define MRLT_UNPACK(...) __VA_ARGS__
+
+template <int D, int M>
+static void project_dm(Launcher& L, int l, int mode)
 {
-    ++n;
-    if (g.d == 1) g.prec ? project_d<1, float>(*this, l, mode) : project_d<1, double>(*this, l, mode);
-    else if (g.d == 2) g.prec ? project_d<2, float>(*this, l, mode) : project_d<2, double>(*this, l, mode);
-    else g.prec ? project_d<3, float>(*this, l, mode) : project_d<3, double>(*this, l, mode);
+    MRLT_T_LAUNCH(L, blocks_list(L.g, l), (L.g, l, mode), k_project<D, M);
+    ++L.n;
 }
+
+void Launcher::project(int l, int mode) { MRLT_DM_DISPATCH(project_dm, *this, l, mode); }
 
 // Up-sweep hi -> lo in groups of at most 6 / d + 1 levels per launch: a group
 // [glo, ghi] has 2^{d (ghi - glo)} <= 64 descendants per top node, so two top
 // nodes fit the NTHREADS = 128 threads of a CTA.
-template <int D, class T>
-static void project_up_d(Launcher& L, int hi, int lo, int mode)
+template <int D, int M>
+static void project_up_dm(Launcher& L, int hi, int lo, int mode)
 {
     constexpr int kDepth = 6 / D;
     static_assert((1 << (D * kDepth)) * 2 <= NTHREADS, "two top nodes per CTA");
     for (int ghi = hi; ghi >= lo;) {
         const int glo = ghi - kDepth > lo ? ghi - kDepth : lo;
         if (glo == ghi) {
-            project_d<D, T>(L, ghi, mode);
+            project_dm<D, M>(L, ghi, mode);
         } else {
             const int tops = NTHREADS >> (D * (ghi - glo));
             long long b = (L.g.N[glo] + tops - 1) / tops;
             if (b > 1216) b = 1216;
-            pdl_launch(k_project_up<D, T>, (int)b, NTHREADS, 0, L.st, L.g, ghi, glo, mode);
+            MRLT_T_LAUNCH(L, (int)b, (L.g, ghi, glo, mode), k_project_up<D, M);
+            ++L.n;
         }
-        ++L.n;
         ghi = glo - 1;
     }
 }
 
 void Launcher::project_up(int hi, int lo, int mode)
 {
-    if (hi < lo) return;
-    if (g.d == 1) g.prec ? project_up_d<1, float>(*this, hi, lo, mode) : project_up_d<1, double>(*this, hi, lo, mode);
-    else if (g.d == 2) g.prec ? project_up_d<2, float>(*this, hi, lo, mode) : project_up_d<2, double>(*this, hi, lo, mode);
-    else g.prec ? project_up_d<3, float>(*this, hi, lo, mode) : project_up_d<3, double>(*this, hi, lo, mode);
+    if (hi >= lo) MRLT_DM_DISPATCH(project_up_dm, *this, hi, lo, mode);
 }
 
-template <class T>
-static void leaf_copy_t(Launcher& L, int lo, int hi, int from, int to)
+template <int D, int M>
+static void leaf_copy_dm(Launcher& L, int lo, int hi, int from, int to)
 {
-    pdl_launch(k_leaf_copy<T>, blocks_list(L.g, hi), NTHREADS, 0, L.st, L.g, lo, hi, from, to);
+    MRLT_T_LAUNCH(L, blocks_list(L.g, hi), (L.g, lo, hi, from, to), k_leaf_copy<M);
+    ++L.n;
 }
 
-void Launcher::leaf_copy(int lo, int hi, int from, int to)
-{
-    ++n;
-    MRLT_T_DISPATCH(leaf_copy_t, *this, lo, hi, from, to);
-}
+void Launcher::leaf_copy(int lo, int hi, int from, int to) { MRLT_DM_DISPATCH(leaf_copy_dm, *this, lo, hi, from, to); }
 
 template <int D, int M>
 static void adapt_dm(Launcher& L, int la, long long it)
@@ -343,16 +340,6 @@ static void apply_dm(Launcher& L, int la)
     }
 }
 
-#define MRLT_DM_DISPATCH(fn, ...)                                   \
-    do {                                                            \
-        if (g.d == 1 && g.m == 1) fn<1, 1>(__VA_ARGS__);            \
-        else if (g.d == 1) fn<1, 3>(__VA_ARGS__);                   \
-        else if (g.d == 2 && g.m == 1) fn<2, 1>(__VA_ARGS__);       \
-        else if (g.d == 2) fn<2, 4>(__VA_ARGS__);                   \
-        else if (g.m == 1) fn<3, 1>(__VA_ARGS__);                   \
-        else fn<3, 5>(__VA_ARGS__);                                 \
-    } while (0)
-
 void Launcher::mark_refinements(int la, long long it) { MRLT_DM_DISPATCH(adapt_dm, *this, la, it); }
 void Launcher::apply_tree(int la) { MRLT_DM_DISPATCH(apply_dm, *this, la); }
 
@@ -365,20 +352,14 @@ void Launcher::compact(int lo, int hi)
     n += 2;
 }
 
-template <class T>
-static void reflux_t(Launcher& L, int lo, int hi)
+template <int D, int M>
+static void reflux_dm(Launcher& L, int lo, int hi)
 {
-    const Grid& g = L.g;
-    if (g.d == 1) pdl_launch(k_reflux<1, T>, blocks_list(g, hi), NTHREADS, 0, L.st, g, lo, hi);
-    else if (g.d == 2) pdl_launch(k_reflux<2, T>, blocks_list(g, hi), NTHREADS, 0, L.st, g, lo, hi);
-    else pdl_launch(k_reflux<3, T>, blocks_list(g, hi), NTHREADS, 0, L.st, g, lo, hi);
+    MRLT_T_LAUNCH(L, blocks_list(L.g, hi), (L.g, lo, hi), k_reflux<D, M);
+    ++L.n;
 }
 
-void Launcher::reflux(int lo, int hi)
-{
-    ++n;
-    MRLT_T_DISPATCH(reflux_t, *this, lo, hi);
-}
+void Launcher::reflux(int lo, int hi) { MRLT_DM_DISPATCH(reflux_dm, *this, lo, hi); }
 
 __global__ void k_scale_init(Grid g)
 {
@@ -563,30 +544,34 @@ void Launcher::set_dt(double dt)
     ++n;
 }
 
-void Launcher::scale(int l)
+template <int D, int M>
+static void scale_dm(Launcher& L)
 {
-    ++n;
-    if (g.prec) k_scale<float><<<blocks_list(g, l), NTHREADS, 0, st>>>(g, l);
-    else k_scale<double><<<blocks_list(g, l), NTHREADS, 0, st>>>(g, l);
+    MRLT_T_LAUNCH(L, blocks_list(L.g, L.g.L), (L.g), k_scale<M);
+    ++L.n;
 }
-void Launcher::finite(int l)
+void Launcher::scale() { MRLT_DM_DISPATCH(scale_dm, *this); }
+
+template <int D, int M>
+static void finite_dm(Launcher& L)
 {
-    ++n;
-    if (g.prec) k_finite<float><<<blocks_list(g, l), NTHREADS, 0, st>>>(g, l);
-    else k_finite<double><<<blocks_list(g, l), NTHREADS, 0, st>>>(g, l);
+    MRLT_T_LAUNCH(L, blocks_list(L.g, L.g.L), (L.g), k_finite<M);
+    ++L.n;
 }
+void Launcher::finite() { MRLT_DM_DISPATCH(finite_dm, *this); }
 void Launcher::mass(int l, double* part)
 {
     ++n;
     if (g.prec) k_mass<float><<<MASS_BLOCKS, NTHREADS, 0, st>>>(g, l, part);
     else k_mass<double><<<MASS_BLOCKS, NTHREADS, 0, st>>>(g, l, part);
 }
-void Launcher::pack(int l, long long base, int* keys, double* vals)
+template <int D, int M>
+static void pack_dm(Launcher& L, int* keys, double* vals)
 {
-    ++n;
-    if (g.prec) k_pack<float><<<blocks_list(g, l), NTHREADS, 0, st>>>(g, l, base, keys, vals);
-    else k_pack<double><<<blocks_list(g, l), NTHREADS, 0, st>>>(g, l, base, keys, vals);
+    MRLT_T_LAUNCH(L, blocks_list(L.g, L.g.L), (L.g, keys, vals), k_pack<M);
+    ++L.n;
 }
+void Launcher::pack(int* keys, double* vals) { MRLT_DM_DISPATCH(pack_dm, *this, keys, vals); }
 void Launcher::uniform(double* T, uint8_t* us)
 {
     for (int l = g.L; l >= g.lb; --l, ++n) {

@@ -19,7 +19,7 @@ struct Launcher {
     void apply_tree(int la);
     void compact(int lo, int hi);                      // leaf / node / tile lists of levels lo..hi
     void reflux(int lo, int hi);                       // coarse levels lo..hi
-    void scale(int l);
+    void scale();                                      // running max |q_v| over all leaves
     void scale_init();                                 // running max |q_v| := 1e-14
     void set_dt(double dt);                            // *g.dtp := dt
     void set_leaves(const int* keys, const double* vals, long long count); // leaf q^n and end values
@@ -28,9 +28,9 @@ struct Launcher {
     // compacting copy of the nodes from `from` into the arrays of g (a new capacity)
     void renumber(const Grid& from, const int* counts_host, long long used);
     void count_refined(int la, int* out);   // *out = refinement flags of levels la..L-1
-    void finite(int l);
+    void finite();                                     // all leaves
     void mass(int l, double* part);
-    void pack(int l, long long base, int* keys, double* vals);
+    void pack(int* keys, double* vals);                // all leaves, in level and list order
     void uniform(double* T, uint8_t* us);
 };
 

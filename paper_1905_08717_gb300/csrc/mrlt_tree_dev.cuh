@@ -16,29 +16,92 @@ enum ProjMode { PM_Q0 = 0, PM_Q1, PM_Q2, PM_REF2, PM_PRJ2, PM_REF3, PM_PRJ3, PM_
 #define MRLT_GRID_STRIDE(i, n) \
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < (n); i += (long long)gridDim.x * blockDim.x)
 
-// ------------------------------------------------------------ simple leaf copies
+// ------------------------------------------------------------ lists and rows
+// f(l, id, t) for every entry of the leaf lists (KIND 0) or internal-node
+// lists (KIND 1) of levels lo..hi, level by level as one range t = 0, 1, ...
+// over the launch's threads: one pass whatever the number of levels, where a
+// loop over the levels costs a chain of dependent loads for each.  Every thread
+// of the CTA takes part.
+template <int KIND, class F>
+__device__ __forceinline__ void for_list(const Grid& g, int lo, int hi, F f)
+{
+    __shared__ int base[LMAX + 2]; // level lo + k starts at base[k]
+    __syncthreads();               // base may hold an earlier call's
+    if (threadIdx.x < 32) {
+        const int k = threadIdx.x, n = hi - lo + 1;
+        int inc = k < n ? g.counts[KIND * (LMAX + 1) + lo + k] : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int x = __shfl_up_sync(0xffffffffu, inc, o);
+            if (k >= o) inc += x;
+        }
+        if (k < n) base[k + 1] = inc;
+        if (k == 0) base[0] = 0;
+    }
+    __syncthreads();
+    const int* list = KIND ? g.inner : g.leaves;
+    const int total = base[hi - lo + 1];
+    MRLT_GRID_STRIDE(t, total)
+    {
+        int k = hi - lo; // most entries are on the finest levels
+        while (t < base[k]) --k;
+        const long long id = list[g.off[lo + k] + t - base[k]];
+        if (id < 0 || id >= g.N[lo + k]) {
+            atomicOr(g.err, ERR_INDEX);
+            continue;
+        }
+        f(lo + k, id, t);
+    }
+}
+
+// product rounded by itself (never contracted into a multiply-add)
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
+// a node's row of M values: 16-byte accesses where rows are whole vectors
+template <int M, class T>
+__device__ __forceinline__ void load_row(const T* p, T (&r)[M])
+{
+    if constexpr (M * sizeof(T) % 16 == 0) {
+        constexpr int E = 16 / sizeof(T);
+#pragma unroll
+        for (int k = 0; k < M / E; ++k) {
+            const int4 x = reinterpret_cast<const int4*>(p)[k];
+            memcpy(&r[k * E], &x, 16);
+        }
+    } else {
+#pragma unroll
+        for (int v = 0; v < M; ++v) r[v] = p[v];
+    }
+}
+template <int M, class T>
+__device__ __forceinline__ void store_row(T* p, const T (&r)[M])
+{
+    if constexpr (M * sizeof(T) % 16 == 0) {
+        constexpr int E = 16 / sizeof(T);
+#pragma unroll
+        for (int k = 0; k < M / E; ++k) {
+            int4 x;
+            memcpy(&x, &r[k * E], 16);
+            reinterpret_cast<int4*>(p)[k] = x;
+        }
+    } else {
+#pragma unroll
+        for (int v = 0; v < M; ++v) p[v] = r[v];
+    }
+}
+
 // T: storage type of the fields (double, or float in the mixed mode); the
 // arithmetic of a body is in T except where it says otherwise
-template <class T>
+template <int M, class T>
 __device__ __forceinline__ void dev_leaf_copy(const Grid& g, int lo, int hi, int from, int to)
 {
-    for (int l = lo; l <= hi; ++l) {
-        const int cnt = g.counts[l];
-        const int* list = g.leaves + g.off[l];
-        const long long N = g.N[l];
-        MRLT_GRID_STRIDE(t, cnt)
-        {
-            const long long id = list[t];
-            if (id < 0 || id >= N) {
-                atomicOr(g.err, ERR_INDEX);
-                continue;
-            }
-            const int sl = slot_of(g, l, id);
-            const T* a = nd<T>(g, from, sl);
-            T* b = nd<T>(g, to, sl);
-            for (int v = 0; v < g.m; ++v) b[v] = a[v];
-        }
-    }
+    for_list<0>(g, lo, hi, [&](int l, long long id, long long) {
+        const int sl = slot_of(g, l, id);
+        T r[M];
+        load_row<M, T>(nd<T>(g, from, sl), r);
+        store_row<M, T>(nd<T>(g, to, sl), r);
+    });
 }
 
 // ------------------------------------------------------------ projections
@@ -50,8 +113,14 @@ __device__ __forceinline__ void dev_leaf_copy(const Grid& g, int lo, int hi, int
 //  PM_PRJ3: Alg. 6 -- q** = mean(children at t^n + dt_{l+1}), end value
 //           2 q** - q^n (Eq. 16 with the theta values implied by q**)
 //  PM_MID:  Alg. 3 / Sec. 4.3 refresh of the mid-step level lmin-1
-// one internal node (l, id): the projection of the given mode
-template <int D, class T>
+// one internal node (l, id): the projection of the given mode.  Bound by its
+// dependent trips (list, child slots, rows), so the rows of all children are
+// loaded before any is used; a loop over the variables that stored each before
+// loading the next took 8.8 us per launch over the opening of the 2D Euler
+// L = 10 solve on a GB300 (14 k nodes on level 9), this takes 6.0 us.  The
+// roundings are written out: which multiply-adds are fused must not depend on
+// what else the compiler finds to share.
+template <int D, int M, class T>
 __device__ __forceinline__ void project_node(const Grid& g, int l, long long id, int mode)
 {
     constexpr int NCH = 1 << D;
@@ -67,84 +136,97 @@ __device__ __forceinline__ void project_node(const Grid& g, int l, long long id,
         csl[k] = slot_of(g, l + 1, ch);
     }
     const int sl = slot_of(g, l, id);
-    T* q0 = nd<T>(g, F_Q0, sl);
-    T* q1 = nd<T>(g, F_Q1, sl);
-    T* q2 = nd<T>(g, F_Q2, sl);
-    T* qe = nd<T>(g, F_QE, sl);
-    for (int v = 0; v < g.m; ++v) {
-        const int o = v;
-        T acc = T(0);
+    const int child = mode == PM_Q1 || mode == PM_REF2   ? F_Q1
+                      : mode == PM_Q2 || mode == PM_REF3 ? F_Q2
+                      : mode == PM_PRJ3                  ? F_QE
+                                                         : F_Q0; // PM_Q0; PM_MID: children at t^n
+    T w[NCH][M], acc[M], a0[M], a1[M];
+    if (mode == PM_PRJ2) {
+        T x[NCH][M];
 #pragma unroll
         for (int k = 0; k < NCH; ++k) {
-            const T* c0 = nd<T>(g, F_Q0, csl[k]);
-            const T* c1 = nd<T>(g, F_Q1, csl[k]);
-            const T* c2 = nd<T>(g, F_Q2, csl[k]);
-            const T* ce = nd<T>(g, F_QE, csl[k]);
-            const int oc = v;
-            T w;
-            switch (mode) {
-            case PM_Q0: w = c0[oc]; break;
-            case PM_Q1: case PM_REF2: w = c1[oc]; break;
-            case PM_Q2: case PM_REF3: w = c2[oc]; break;
-            case PM_PRJ2:
-                if (cst[k] == 1) w = g.rk == 2 ? T(2) * ce[oc] - c0[oc] : T(4) * c2[oc] - T(3) * c0[oc];
-                else w = T(2) * c1[oc] - c0[oc];
-                break;
-            case PM_PRJ3: w = ce[oc]; break;
-            default: w = c0[oc]; break; // PM_MID: children at t^n
+            load_row<M, T>(nd<T>(g, F_Q0, csl[k]), w[k]);
+            load_row<M, T>(nd<T>(g, cst[k] != 1 ? F_Q1 : (g.rk == 2 ? F_QE : F_Q2), csl[k]), x[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < NCH; ++k)
+#pragma unroll
+            for (int v = 0; v < M; ++v) {
+                if (cst[k] == 1 && g.rk != 2) w[k][v] = fma(T(4), x[k][v], -mul_rn(T(3), w[k][v]));
+                else w[k][v] = T(2) * x[k][v] - w[k][v];
             }
-            acc += w;
+    } else {
+#pragma unroll
+        for (int k = 0; k < NCH; ++k) load_row<M, T>(nd<T>(g, child, csl[k]), w[k]);
+        if (mode >= PM_REF2) {
+            load_row<M, T>(nd<T>(g, F_Q0, sl), a0);
+            if (mode == PM_REF3 || mode == PM_MID) load_row<M, T>(nd<T>(g, F_Q1, sl), a1);
         }
-        const T mean = acc * T(1.0 / NCH);
-        switch (mode) {
-        case PM_Q0: q0[o] = mean; break;
-        case PM_Q1: case PM_PRJ2: q1[o] = mean; break;
-        case PM_Q2: q2[o] = mean; break;
-        case PM_REF2:
-            nd<T>(g, F_XH, sl)[o] = mean;
-            q1[o] = T(2) * mean - q0[o];
-            break;
-        case PM_REF3: {
-            nd<T>(g, F_N1, sl)[o] = mean;
-            nd<T>(g, F_N3, sl)[o] = T(-6.5) * q0[o] - T(1.5) * q1[o] + T(9) * mean;
-            q2[o] = T(-5.5) * q0[o] - T(1.5) * q1[o] + T(8) * mean;
-            break;
-        }
-        case PM_PRJ3:
-            q2[o] = mean;
-            qe[o] = T(2) * mean - q0[o];
-            break;
-        default: { // PM_MID
-            if (g.rk == 2) {
-                nd<T>(g, F_NH, sl)[o] = mean;
-                qe[o] = T(-2) * q0[o] - q1[o] + T(4) * mean;
-            } else {
-                q2[o] = mean;
-                qe[o] = T(2) * mean - q0[o];
-                const T n1 = (mean + T(5.5) * q0[o] + T(1.5) * q1[o]) * T(0.125);
-                nd<T>(g, F_N1, sl)[o] = n1;
-                nd<T>(g, F_N3, sl)[o] = T(-6.5) * q0[o] - T(1.5) * q1[o] + T(9) * n1;
+    }
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+        acc[v] = T(0);
+#pragma unroll
+        for (int k = 0; k < NCH; ++k) acc[v] += w[k][v];
+        acc[v] = acc[v] * T(1.0 / NCH); // the mean
+    }
+    switch (mode) {
+    case PM_Q0: store_row<M, T>(nd<T>(g, F_Q0, sl), acc); break;
+    case PM_Q1: case PM_PRJ2: store_row<M, T>(nd<T>(g, F_Q1, sl), acc); break;
+    case PM_Q2: store_row<M, T>(nd<T>(g, F_Q2, sl), acc); break;
+    case PM_REF2:
+        store_row<M, T>(nd<T>(g, F_XH, sl), acc);
+#pragma unroll
+        for (int v = 0; v < M; ++v) acc[v] = T(2) * acc[v] - a0[v];
+        store_row<M, T>(nd<T>(g, F_Q1, sl), acc);
+        break;
+    case PM_REF3: {
+        T r[M];
+        store_row<M, T>(nd<T>(g, F_N1, sl), acc);
+#pragma unroll
+        for (int v = 0; v < M; ++v) r[v] = fma(T(9), acc[v], fma(T(-6.5), a0[v], -mul_rn(T(1.5), a1[v])));
+        store_row<M, T>(nd<T>(g, F_N3, sl), r);
+#pragma unroll
+        for (int v = 0; v < M; ++v) r[v] = fma(T(8), acc[v], fma(T(-5.5), a0[v], -mul_rn(T(1.5), a1[v])));
+        store_row<M, T>(nd<T>(g, F_Q2, sl), r);
+        break;
+    }
+    case PM_PRJ3:
+        store_row<M, T>(nd<T>(g, F_Q2, sl), acc);
+#pragma unroll
+        for (int v = 0; v < M; ++v) acc[v] = T(2) * acc[v] - a0[v];
+        store_row<M, T>(nd<T>(g, F_QE, sl), acc);
+        break;
+    default: { // PM_MID
+        T r[M];
+        if (g.rk == 2) {
+            store_row<M, T>(nd<T>(g, F_NH, sl), acc);
+#pragma unroll
+            for (int v = 0; v < M; ++v) r[v] = T(-2) * a0[v] - a1[v] + T(4) * acc[v];
+            store_row<M, T>(nd<T>(g, F_QE, sl), r);
+        } else {
+            T n1[M];
+            store_row<M, T>(nd<T>(g, F_Q2, sl), acc);
+#pragma unroll
+            for (int v = 0; v < M; ++v) {
+                r[v] = T(2) * acc[v] - a0[v];
+                n1[v] = fma(T(1.5), a1[v], fma(T(5.5), a0[v], acc[v])) * T(0.125);
             }
+            store_row<M, T>(nd<T>(g, F_QE, sl), r);
+            store_row<M, T>(nd<T>(g, F_N1, sl), n1);
+#pragma unroll
+            for (int v = 0; v < M; ++v)
+                r[v] = fma(T(9), n1[v], fma(T(-6.5), a0[v], -mul_rn(T(1.5), a1[v])));
+            store_row<M, T>(nd<T>(g, F_N3, sl), r);
         }
-        }
+    }
     }
 }
 
-template <int D, class T>
+template <int D, int M, class T>
 __device__ __forceinline__ void dev_project(const Grid& g, int l, int mode)
 {
-    const int cnt = g.counts[LMAX + 1 + l];
-    const int* list = g.inner + g.off[l];
-    const long long N = g.N[l];
-    MRLT_GRID_STRIDE(t, cnt)
-    {
-        const long long id = list[t];
-        if (id < 0 || id >= N) {
-            atomicOr(g.err, ERR_INDEX);
-            continue;
-        }
-        project_node<D, T>(g, l, id, mode);
-    }
+    for_list<1>(g, l, l, [&](int, long long id, long long) { project_node<D, M, T>(g, l, id, mode); });
 }
 
 // An up-sweep of one mode over levels hi..lo (hi - lo = depth >= 1) in one
@@ -155,7 +237,7 @@ __device__ __forceinline__ void dev_project(const Grid& g, int l, int mode)
 // of top node t / sub on each level (sub = 2^{d (m - lo)} on level m), so
 // 2^{d depth} <= blockDim.x is required.  Every node is projected by the same
 // operations as in dev_project.
-template <int D, class T>
+template <int D, int M, class T>
 __device__ __forceinline__ void dev_project_up(const Grid& g, int hi, int lo, int mode)
 {
     const int depth = hi - lo;
@@ -165,8 +247,8 @@ __device__ __forceinline__ void dev_project_up(const Grid& g, int hi, int lo, in
     const long long N = g.N[lo];
     const int nstep = (cnt + tops - 1) / tops;
     for (int c = blockIdx.x; c < nstep; c += gridDim.x) { // uniform across the CTA
-        for (int m = hi; m >= lo; --m) {
-            const int s = m - lo;
+        for (int u = hi; u >= lo; --u) {
+            const int s = u - lo;
             const int sub = 1 << (D * s);
             const int t = threadIdx.x;
             const int ti = c * tops + t / sub;
@@ -178,10 +260,10 @@ __device__ __forceinline__ void dev_project_up(const Grid& g, int hi, int lo, in
                     int tc[3];
                     cell_xyz(g, lo, top, tc);
                     const int r = t % sub, msk = (1 << s) - 1;
-                    const long long id = cell_id(g, m, (tc[0] << s) + (r & msk),
+                    const long long id = cell_id(g, u, (tc[0] << s) + (r & msk),
                                                  D > 1 ? (tc[1] << s) + ((r >> s) & msk) : 0,
                                                  D > 2 ? (tc[2] << s) + (r >> (2 * s)) : 0);
-                    if (status(g, m, id) == 2) project_node<D, T>(g, m, id, mode);
+                    if (status(g, u, id) == 2) project_node<D, M, T>(g, u, id, mode);
                 }
             }
             __syncthreads();
@@ -941,113 +1023,117 @@ __device__ __forceinline__ void level_tile_list(const Grid& g, int l)
 }
 
 // ------------------------------------------------------------ registers
-// conservative correction of the coarse leaves of level l whose step ended:
-// q += +-(coarse time-integrated flux - mean of the fine ones) / dx; the
-// registers read are cleared for the next step
-template <int D, class T>
+// conservative correction of the coarse leaves of levels lo..hi whose step
+// ended: q += +-(coarse time-integrated flux - mean of the fine ones) / dx; the
+// registers read are cleared for the next step.  Bound by the dependent trips
+// of a leaf (neighbours' statuses, children's slots, registers), so each trip
+// loads all it can: the statuses of all faces at once, the rows of a face's
+// children at once.  One face, variable and child after the other took 40 us
+// per launch over the opening of the 2D Euler L = 10 solve on a GB300 (73 k
+// leaves), and 142 us in the 3D blast at L = 7; this takes 13 and 36 us.
+template <int D, int M, class T>
 __device__ __forceinline__ void dev_reflux(const Grid& g, int lo, int hi)
 {
-    for (int l = lo; l <= hi; ++l) {
-        const int cnt = g.counts[l];
-        const int* list = g.leaves + g.off[l];
-        const long long N = g.N[l];
-        const int m = g.m;
-        constexpr int NT = 1 << (D - 1);
-        MRLT_GRID_STRIDE(t, cnt)
-        {
-            const long long id = list[t];
-            if (id < 0 || id >= N) {
-                atomicOr(g.err, ERR_INDEX);
-                continue;
-            }
-            int c[3];
-            cell_xyz(g, l, id, c);
-            for (int fi = 0; fi < 2 * D; ++fi) {
-                const int k = fi >> 1, side = (fi & 1) ? 1 : -1;
-                int q;
-                if (!in_box(g, l, k, c[k] + side, &q)) continue;
-                int nb[3] = {c[0], c[1], c[2]};
-                nb[k] = q;
-                if (status(g, l, cell_id(g, l, nb[0], nb[1], nb[2])) != 2) continue;
-                const int opp = 2 * k + (side > 0 ? 0 : 1);
-                long long ch[NT];
-                for (int tt = 0; tt < NT; ++tt) {
-                    int p[3] = {0, 0, 0}, bit = 0;
-                    for (int j = 0; j < D; ++j) {
-                        if (j == k) continue;
-                        p[j] = 2 * nb[j] + ((tt >> bit) & 1);
-                        ++bit;
-                    }
-                    p[k] = 2 * nb[k] + (side > 0 ? 0 : 1);
-                    ch[tt] = cell_id(g, l + 1, p[0], p[1], p[2]);
-                    if (status(g, l + 1, ch[tt]) != 1) atomicOr(g.err, ERR_REFLUX);
-                }
-                const int sl = slot_of(g, l, id);
-                double* rc = regs(g.rg, g, sl);
-                int csl[NT];
-                for (int tt = 0; tt < NT; ++tt) csl[tt] = slot_of(g, l + 1, ch[tt]);
-                T* qe = nd<T>(g, F_QE, sl);
-                const double idx = 1.0 / g.dx[l][k];
-                for (int v = 0; v < m; ++v) {
-                    double sum = 0.0;
-                    for (int tt = 0; tt < NT; ++tt) {
-                        double* r = regs(g.rg, g, csl[tt]) + opp * m + v;
-                        sum += *r;
-                        *r = 0.0;
-                    }
-                    double* r = rc + fi * m + v;
-                    // the correction from the FP64 registers, rounded to T once
-                    qe[v] = T(double(qe[v]) + side * (*r - sum * (1.0 / NT)) * idx);
-                    *r = 0.0;
-                }
-            }
+    constexpr int NT = 1 << (D - 1);
+    for_list<0>(g, lo, hi, [&](int l, long long id, long long) {
+        int c[3];
+        cell_xyz(g, l, id, c);
+        uint8_t st[2 * D];
+#pragma unroll
+        for (int fi = 0; fi < 2 * D; ++fi) {
+            int nb[3] = {c[0], c[1], c[2]};
+            st[fi] = in_box(g, l, fi >> 1, c[fi >> 1] + (fi & 1 ? 1 : -1), &nb[fi >> 1])
+                         ? status(g, l, cell_id(g, l, nb[0], nb[1], nb[2]))
+                         : 0;
         }
-    }
+        unsigned finer = 0; // faces to an internal node
+#pragma unroll
+        for (int fi = 0; fi < 2 * D; ++fi) finer |= (st[fi] == 2 ? 1u : 0u) << fi;
+        if (!finer) return;
+        const int sl = slot_of(g, l, id);
+        double* rc = regs(g.rg, g, sl);
+        T q[M];
+        load_row<M, T>(nd<T>(g, F_QE, sl), q);
+        for (; finer; finer &= finer - 1) {
+            const int fi = __ffs(finer) - 1, k = fi >> 1, side = (fi & 1) ? 1 : -1;
+            const int opp = 2 * k + (side > 0 ? 0 : 1);
+            int nk; // the neighbour's coordinate along k
+            in_box(g, l, k, (k == 0 ? c[0] : (k == 1 ? c[1] : c[2])) + side, &nk);
+            double* rf[NT];
+#pragma unroll
+            for (int tt = 0; tt < NT; ++tt) {
+                int p[3] = {0, 0, 0}, bit = 0;
+#pragma unroll
+                for (int j = 0; j < D; ++j) {
+                    if (j == k) p[j] = 2 * nk + (side > 0 ? 0 : 1);
+                    else p[j] = 2 * c[j] + ((tt >> bit++) & 1);
+                }
+                const long long ch = cell_id(g, l + 1, p[0], p[1], p[2]);
+                if (status(g, l + 1, ch) != 1) atomicOr(g.err, ERR_REFLUX);
+                rf[tt] = regs(g.rg, g, slot_of(g, l + 1, ch)) + opp * M;
+            }
+            double r[NT][M], own[M];
+            const double none[M] = {};
+            load_row<M, double>(rc + fi * M, own);
+#pragma unroll
+            for (int tt = 0; tt < NT; ++tt) load_row<M, double>(rf[tt], r[tt]);
+            const double idx = g.rdx[l][k];
+#pragma unroll
+            for (int v = 0; v < M; ++v) {
+                double sum = 0.0;
+#pragma unroll
+                for (int tt = 0; tt < NT; ++tt) sum += r[tt][v];
+                // the correction from the FP64 registers, rounded to T once
+                q[v] = T(double(q[v]) + side * (own[v] - sum * (1.0 / NT)) * idx);
+            }
+            store_row<M, double>(rc + fi * M, none);
+#pragma unroll
+            for (int tt = 0; tt < NT; ++tt) store_row<M, double>(rf[tt], none);
+        }
+        store_row<M, T>(nd<T>(g, F_QE, sl), q);
+    });
 }
 
 // ------------------------------------------------------------ reductions
+// *at = max(*at, x), for the bit patterns of non-negative doubles; most calls
+// find a larger value already there and skip the atomic
+__device__ __forceinline__ void max_bits(unsigned long long* at, double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    if (b > *(volatile unsigned long long*)at) atomicMax(at, b);
+}
+
 // running max |q^n_v| over the leaves of levels lo..hi (detail normalisation)
-template <class T>
+template <int M, class T>
 __device__ __forceinline__ void dev_scale(const Grid& g, int lo, int hi)
 {
-    for (int l = lo; l <= hi; ++l) {
-        const int cnt = g.counts[l];
-        const int* list = g.leaves + g.off[l];
-        const long long N = g.N[l];
-        double mx[MMAX] = {0.0, 0.0, 0.0, 0.0, 0.0};
-        MRLT_GRID_STRIDE(t, cnt)
-        {
-            const long long id = list[t];
-            if (id < 0 || id >= N) continue;
-            const T* q0 = nd<T>(g, F_Q0, slot_of(g, l, id));
-            for (int v = 0; v < g.m; ++v) mx[v] = fmax(mx[v], fabs(double(q0[v])));
-        }
-        for (int v = 0; v < g.m; ++v) {
-            double a = mx[v];
-            for (int o = 16; o > 0; o >>= 1) a = fmax(a, __shfl_xor_sync(0xffffffffu, a, o));
-            if ((threadIdx.x & 31) == 0 && a > 0.0)
-                atomicMax(&g.scale_bits[v], (unsigned long long)__double_as_longlong(a));
-        }
+    double mx[M] = {};
+    for_list<0>(g, lo, hi, [&](int l, long long id, long long) {
+        T q0[M];
+        load_row<M, T>(nd<T>(g, F_Q0, slot_of(g, l, id)), q0);
+#pragma unroll
+        for (int v = 0; v < M; ++v) mx[v] = fmax(mx[v], fabs(double(q0[v])));
+    });
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+        double a = mx[v];
+        for (int o = 16; o > 0; o >>= 1) a = fmax(a, __shfl_xor_sync(0xffffffffu, a, o));
+        if ((threadIdx.x & 31) == 0 && a > 0.0) max_bits(&g.scale_bits[v], a);
     }
 }
 
 // non-finite end values of the leaves of levels lo..hi set ERR_NONFINITE
-template <class T>
+template <int M, class T>
 __device__ __forceinline__ void dev_finite(const Grid& g, int lo, int hi)
 {
-    for (int l = lo; l <= hi; ++l) {
-        const int cnt = g.counts[l];
-        const int* list = g.leaves + g.off[l];
-        const long long N = g.N[l];
-        MRLT_GRID_STRIDE(t, cnt)
-        {
-            const long long id = list[t];
-            if (id < 0 || id >= N) continue;
-            const T* qe = nd<T>(g, F_QE, slot_of(g, l, id));
-            for (int v = 0; v < g.m; ++v)
-                if (!isfinite(double(qe[v]))) atomicOr(g.err, ERR_NONFINITE);
-        }
-    }
+    for_list<0>(g, lo, hi, [&](int l, long long id, long long) {
+        T qe[M];
+        load_row<M, T>(nd<T>(g, F_QE, slot_of(g, l, id)), qe);
+        bool ok = true;
+#pragma unroll
+        for (int v = 0; v < M; ++v) ok = ok && isfinite(double(qe[v]));
+        if (!ok) atomicOr(g.err, ERR_NONFINITE);
+    });
 }
 
 // largest sum of characteristic speeds over the leaves of levels lo..hi (CFL
@@ -1057,25 +1143,18 @@ __device__ __forceinline__ void dev_wave(const Grid& g, int lo, int hi)
 {
     constexpr int M = EQ == 2 ? D + 2 : 1;
     double w = 0.0;
-    for (int l = lo; l <= hi; ++l) {
-        const int cnt = g.counts[l];
-        const int* list = g.leaves + g.off[l];
-        const long long N = g.N[l];
-        MRLT_GRID_STRIDE(t, cnt)
-        {
-            const long long id = list[t];
-            if (id < 0 || id >= N) continue;
-            const T* qe = nd<T>(g, F_QE, slot_of(g, l, id));
-            double q[M];
+    for_list<0>(g, lo, hi, [&](int l, long long id, long long) {
+        T qe[M];
+        load_row<M, T>(nd<T>(g, F_QE, slot_of(g, l, id)), qe);
+        double q[M];
 #pragma unroll
-            for (int v = 0; v < M; ++v) q[v] = double(qe[v]);
-            const double s = wave_speed<EQ, D, M>(g, q);
-            w = fmax(w, s != s ? 1e300 : s);
-        }
-    }
+        for (int v = 0; v < M; ++v) q[v] = double(qe[v]);
+        const double s = wave_speed<EQ, D, M>(g, q);
+        w = fmax(w, s != s ? 1e300 : s);
+    });
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) w = fmax(w, __shfl_xor_sync(0xffffffffu, w, o));
-    if ((threadIdx.x & 31) == 0 && w > 0.0) atomicMax(g.wmax, (unsigned long long)__double_as_longlong(w));
+    if ((threadIdx.x & 31) == 0 && w > 0.0) max_bits(g.wmax, w);
 }
 
 } // namespace mrlt
