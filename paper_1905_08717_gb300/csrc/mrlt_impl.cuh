@@ -370,55 +370,6 @@ __device__ __forceinline__ void predict(const Grid& g, const Ctx& x, int l, cons
     }
 }
 
-// Predictions (Eq. 4, tensor product) of all 2^d children on level l + 1 of
-// the node at in-box coordinates c of level l: the 3^d block around c is read
-// once and enters every child with that child's weights.  Each child's sum
-// runs over the block in the order of predict(), so out[k] equals
-// predict(g, x, l + 1, 2 c + k) term by term.
-template <int D, int M, class T>
-__device__ __forceinline__ void predict_children(const Grid& g, const Ctx& x, int l, const int c[3],
-                                                 double (*out)[M])
-{
-    constexpr int NCH = 1 << D;
-#pragma unroll
-    for (int k = 0; k < NCH; ++k)
-#pragma unroll
-        for (int v = 0; v < M; ++v) out[k][v] = 0.0;
-#pragma unroll(D > 2 ? 1 : 3)
-    for (int dz = (D > 2 ? -1 : 0); dz <= (D > 2 ? 1 : 0); ++dz) {
-        int nz = 0;
-        const int z = D > 2 ? wrap_or_mirror(g, l, 2, c[2] + dz, nz) : 0;
-#pragma unroll(D > 2 ? 1 : 3)
-        for (int dy = (D > 1 ? -1 : 0); dy <= (D > 1 ? 1 : 0); ++dy) {
-            int nyz = nz;
-            const int y = D > 1 ? wrap_or_mirror(g, l, 1, c[1] + dy, nyz) : 0;
-#pragma unroll
-            for (int dxx = -1; dxx <= 1; ++dxx) {
-                int neg = nyz;
-                const int xx = wrap_or_mirror(g, l, 0, c[0] + dxx, neg);
-                const long long id = cell_id(g, l, xx, y, z);
-                const int st = status(g, l, id);
-                const int sl = slot_of(g, l, id);
-                if (st == 0) {
-                    atomicOr(g.err, ERR_SOURCE);
-                    continue;
-                }
-                double val[M];
-                expose<M, T, double>(g, x, l, sl, st, val);
-#pragma unroll
-                for (int k = 0; k < NCH; ++k) {
-                    const double wz = D > 2 ? pw((k >> 2) & 1, dz) : 1.0;
-                    const double wyz = wz * (D > 1 ? pw((k >> 1) & 1, dy) : 1.0);
-                    const double w0 = wyz * pw(k & 1, dxx);
-                    const double w = neg ? -w0 : w0; // an odd-mirror ghost enters negated
-#pragma unroll
-                    for (int v = 0; v < M; ++v) out[k][v] += w * val[v];
-                }
-            }
-        }
-    }
-}
-
 // value of the cell at (possibly out-of-box) coordinates p on level l
 template <int D, int M, class T, class O>
 __device__ __forceinline__ void value_at(const Grid& g, const Ctx& x, int l, const int p[3], O* out)
