@@ -39,16 +39,15 @@ namespace mrlt {
 constexpr int LMAX = 16;
 constexpr int MMAX = 5;
 constexpr int NTHREADS = 128;
-// tiles of the tiled stage kernel (d = 1: 64 cells; d = 2: 16 x 8; d = 3: 8 x 4 x 4)
-constexpr int kTile1X = 64;
+// tiles of the tiled stage kernel (d = 1: 48 cells; d = 2: 16 x 8; d = 3: 8 x 4 x 4)
+constexpr int kTile1X = 48;
 constexpr int kTile2X = 16, kTile2Y = 8;
 constexpr int kTile3X = 8, kTile3Y = 4, kTile3Z = 4;
 // threads per tile CTA: two per cell (measured: 3D blast L=8 -10 to -13%, 2D
 // Euler L=10 -1.5% against one per cell; four per cell was slower)
-constexpr int kTileThreads1 = 128, kTileThreads2 = 256, kTileThreads3 = 256;
+constexpr int kTileThreads1 = 64, kTileThreads2 = 256, kTileThreads3 = 256;
 
 enum Field { F_Q0 = 0, F_Q1, F_Q2, F_QE, F_XH, F_NH, F_N1, F_N3, NFIELD };
-enum Kind { K_WALL = 0, K_LEAF = 1, K_FINER = 2, K_COARSER = 3 };
 enum FlagBits { FL_SIG = 1, FL_BIG = 2, FL_REF = 16 };
 enum ErrBits { ERR_INDEX = 1, ERR_SOURCE = 2, ERR_NONFINITE = 4, ERR_REFLUX = 8, ERR_TIMEOUT = 16, ERR_CAPACITY = 32 };
 
@@ -389,6 +388,26 @@ __device__ __forceinline__ void value_at(const Grid& g, const Ctx& x, int l, con
 }
 
 // ---------------------------------------------------------------- physics
+// A product and a sum rounded by themselves, never contracted into a
+// multiply-add.  Where an expression could be contracted in two ways, the one
+// meant is written out: the FP32 results must not depend on what the compiler
+// finds around it.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+
+// a[k] for a run-time direction k < D: selects, where an indexed register
+// array would have to live in local memory
+template <int D, class R>
+__device__ __forceinline__ R along(const R* a, int k)
+{
+    R x = a[0];
+    if (D > 1 && k == 1) x = a[1];
+    if (D > 2 && k == 2) x = a[2];
+    return x;
+}
+
 template <class R>
 __device__ __forceinline__ R minmod(R a, R b)
 {
@@ -507,22 +526,27 @@ __device__ __forceinline__ void flux_recon(const Grid& g, int k, double dxf, con
             keR += PR[1 + c] * PR[1 + c];
         }
         const R igm = R(g.igm);
-        UL[D + 1] = PL[D + 1] * igm + h * PL[0] * keL;
-        UR[D + 1] = PR[D + 1] * igm + h * PR[0] * keR;
-        const R unL = PL[1 + k], unR = PR[1 + k];
+        UL[D + 1] = fma(PL[D + 1], igm, mul_rn(h * PL[0], keL));
+        UR[D + 1] = fma(PR[D + 1], igm, mul_rn(h * PR[0], keR));
+        const R unL = along<D>(PL + 1, k), unR = along<D>(PR + 1, k);
         if (g.flux == 1) { // AUSM+
             ausm_plus<D, M, R>(gam, k, PL, PR, UL, UR, F);
             return;
         }
 #pragma unroll
-        for (int v = 0; v < M; ++v) {
-            FL[v] = UL[v] * unL;
-            FR[v] = UR[v] * unR;
+        for (int v = 0; v <= D; ++v) {
+            FL[v] = mul_rn(UL[v], unL);
+            FR[v] = mul_rn(UR[v], unR);
+            if (v == 1 + k) {
+                FL[v] = add_rn(FL[v], PL[D + 1]);
+                FR[v] = add_rn(FR[v], PR[D + 1]);
+            }
         }
-        FL[1 + k] += PL[D + 1];
-        FR[1 + k] += PR[D + 1];
-        FL[D + 1] += PL[D + 1] * unL;
-        FR[D + 1] += PR[D + 1] * unR;
+        // energy flux (E + p) u_n: which product is rounded first differs by
+        // dimension, as FP32 solves have always had it
+        const R eL = UL[D + 1], eR = UR[D + 1], pL = PL[D + 1], pR = PR[D + 1];
+        FL[D + 1] = D == 2 ? fma(eL, unL, mul_rn(pL, unL)) : fma(pL, unL, mul_rn(eL, unL));
+        FR[D + 1] = D == 2 ? fma(eR, unR, mul_rn(pR, unR)) : fma(pR, unR, mul_rn(eR, unR));
         // sound speeds sqrt(gamma p / rho) = gamma p rsqrt(gamma p rho)
         const R gpL = gam * PL[D + 1], gpR = gam * PR[D + 1];
         const R cL = gpL * rsqrt(gpL * PL[0]);
@@ -538,19 +562,9 @@ __device__ __forceinline__ void flux_recon(const Grid& g, int k, double dxf, con
         } else {
             const R ids = R(1) / (sR - sL);
 #pragma unroll
-            for (int v = 0; v < M; ++v) F[v] = (sR * FL[v] - sL * FR[v] + sL * sR * (UR[v] - UL[v])) * ids;
+            for (int v = 0; v < M; ++v)
+                F[v] = fma(sL * sR, UR[v] - UL[v], fma(sR, FL[v], -mul_rn(sL, FR[v]))) * ids;
         }
-    }
-}
-
-template <int EQ, int M, class R>
-__device__ __forceinline__ void source(const Grid& g, const R* q, R* S)
-{
-#pragma unroll
-    for (int v = 0; v < M; ++v) S[v] = R(0);
-    if constexpr (EQ == 3) {
-        const R u = q[0];
-        S[0] = R(g.phys[1]) * u * (R(1) - u) * (u - R(g.phys[2]));
     }
 }
 

@@ -54,10 +54,6 @@ __device__ __forceinline__ void for_list(const Grid& g, int lo, int hi, F f)
     }
 }
 
-// product rounded by itself (never contracted into a multiply-add)
-__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
-__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
-
 // a node's row of M values: 16-byte accesses where rows are whole vectors
 template <int M, class T>
 __device__ __forceinline__ void load_row(const T* p, T (&r)[M])
