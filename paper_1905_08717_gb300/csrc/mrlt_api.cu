@@ -1004,6 +1004,7 @@ mr_status layout_alloc(mr_solver* h, const mr_config* cfg)
     g.prec = cfg->precision;
     g.flux = cfg->flux;
     g.igm = cfg->equation == MR_EQ_EULER ? 1.0 / (cfg->phys[0] - 1.0) : 0.0;
+    g.cstar = cfg->equation == MR_EQ_EULER ? 2.0 * (cfg->phys[0] - 1.0) / (cfg->phys[0] + 1.0) : 0.0;
     g.gcap = 0;
     long long off = 0, toff = 0;
     h->ntot = 0;

@@ -89,6 +89,7 @@ struct Grid {
     int prec;                       // 0 FP64, 1 mixed: state, fluxes and stage updates in FP32
     int flux;                       // Euler: 0 HLL, 1 AUSM+
     double igm;                     // Euler: 1 / (gamma - 1)
+    double cstar;                   // Euler: 2 (gamma - 1) / (gamma + 1)
     int gcap;                       // CTAs per stage launch at most (0: resident capacity)
 };
 
@@ -311,6 +312,14 @@ __device__ __forceinline__ void expose(const Grid& g, const Ctx& x, int l, int s
     }
 }
 
+// Eq. 4 along one direction in FP64: the child of offset a (0 left, 1 right) of
+// m between its neighbours l and r.  Predictions in FP64 apply it direction by
+// direction (2 operations each) instead of weighting every cell of the block.
+__device__ __forceinline__ double child(double l, double m, double r, int a)
+{
+    return fma(a ? 0.125 : -0.125, r - l, m);
+}
+
 // 1D prediction weights of Eq. 4 for child offset a (0 left, 1 right):
 // child = parent + s (right - left) / 8, s = -1 for a = 0, +1 for a = 1.
 __device__ __forceinline__ double pw(int a, int delta)
@@ -388,6 +397,22 @@ __device__ __forceinline__ void value_at(const Grid& g, const Ctx& x, int l, con
 }
 
 // ---------------------------------------------------------------- physics
+// FP64 operations issue at 2 lanes per clock and SM on this GPU (one warp
+// instruction every 16 cycles), integer operations at 64: comparisons, signs and
+// selections of doubles are done on their bit patterns below.
+__device__ __forceinline__ long long ordered_bits(double a) // ordered as the values are (-0 below +0)
+{
+    const long long x = __double_as_longlong(a);
+    return x ^ (x >> 63 & 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ bool less(double a, double b) { return ordered_bits(a) < ordered_bits(b); }
+__device__ __forceinline__ bool negative(double a) { return __double2hiint(a) < 0; } // sign bit
+__device__ __forceinline__ bool positive(double a) { return __double_as_longlong(a) > 0; } // and not +0
+__device__ __forceinline__ bool below_abs(double a, double b) // |a| < |b|
+{
+    return (__double_as_longlong(a) & 0x7fffffffffffffffLL) < (__double_as_longlong(b) & 0x7fffffffffffffffLL);
+}
+
 // A product and a sum rounded by themselves, never contracted into a
 // multiply-add.  Where an expression could be contracted in two ways, the one
 // meant is written out: the FP32 results must not depend on what the compiler
@@ -396,6 +421,18 @@ __device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, 
 __device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ float add_rn(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(a, b); }
+
+template <class R>
+__device__ __forceinline__ R minmod(R a, R b)
+{
+    if (a * b <= R(0)) return R(0);
+    return fabs(a) < fabs(b) ? a : b;
+}
+__device__ __forceinline__ double minmod(double a, double b)
+{
+    const double m = below_abs(a, b) ? a : b;
+    return (__double2hiint(a) ^ __double2hiint(b)) < 0 ? 0.0 : m;
+}
 
 // a[k] for a run-time direction k < D: selects, where an indexed register
 // array would have to live in local memory
@@ -406,13 +443,6 @@ __device__ __forceinline__ R along(const R* a, int k)
     if (D > 1 && k == 1) x = a[1];
     if (D > 2 && k == 2) x = a[2];
     return x;
-}
-
-template <class R>
-__device__ __forceinline__ R minmod(R a, R b)
-{
-    if (a * b <= R(0)) return R(0);
-    return fabs(a) < fabs(b) ? a : b;
 }
 
 // Variables that MUSCL reconstructs: primitives (rho, u_1..u_d, p) for Euler,
@@ -441,8 +471,8 @@ __device__ __forceinline__ void recon_vars(const Grid& g, const WT* W, R* P)
 }
 
 // AUSM+ (Liou 1996), the paper's Euler flux (Sec. 5), across a face normal
-// to direction k, from the reconstructed primitives (rho, u_1..u_d, p) and
-// conservative states of both sides.  With total enthalpy H = (E + p)/rho
+// to direction k, from the reconstructed primitives (rho, u_1..u_d, p) of both
+// sides.  With total enthalpy H = (E + p)/rho
 // and critical speed a*^2 = 2 (g-1)/(g+1) H, the interface speed is
 // a = min(a*_L^2 / max(a*_L, u_L), a*_R^2 / max(a*_R, -u_R)); the Mach
 // numbers M = u/a are split as M+-(M) = +-(M +- 1)^2/4 +- (M^2 - 1)^2/8 and
@@ -466,12 +496,12 @@ __device__ __forceinline__ R ausm_split_pres(R M, R sgn)
     return R(0.25) * (M + sgn) * (M + sgn) * (R(2) - sgn * M) + sgn * R(0.1875) * M * t * t;
 }
 
-template <int D, int M, class R>
+template <int D, class R>
 __device__ __forceinline__ void ausm_plus(R gam, int k, const R* PL, const R* PR, const R* UL, const R* UR, R* F)
 {
     const R pL = PL[D + 1], pR = PR[D + 1];
     const R HL = (UL[D + 1] + pL) / PL[0], HR = (UR[D + 1] + pR) / PR[0];
-    const R uL = PL[1 + k], uR = PR[1 + k];
+    const R uL = along<D>(PL + 1, k), uR = along<D>(PR + 1, k);
     const R cst = R(2) * (gam - R(1)) / (gam + R(1));
     const R asL = sqrt(cst * HL), asR = sqrt(cst * HR);
     const R atL = asL * asL / fmax(asL, uL);
@@ -483,9 +513,110 @@ __device__ __forceinline__ void ausm_plus(R gam, int k, const R* PL, const R* PR
     const R mp = fmax(mh, R(0)), mm = fmin(mh, R(0));
     F[0] = a * (mp * PL[0] + mm * PR[0]);
 #pragma unroll
-    for (int c = 0; c < D; ++c) F[1 + c] = a * (mp * UL[1 + c] + mm * UR[1 + c]);
+    for (int c = 0; c < D; ++c) {
+        F[1 + c] = mul_rn(a, mp * UL[1 + c] + mm * UR[1 + c]);
+        if (c == k) F[1 + c] = add_rn(F[1 + c], ph);
+    }
     F[D + 1] = a * (mp * (PL[0] * HL) + mm * (PR[0] * HR));
-    F[1 + k] += ph;
+}
+
+// The same in FP64 with fewer operations: three divisions instead of six (a*^2
+// / a* = a* unless the normal flow is above critical; one reciprocal of the
+// interface speed), the polynomials of a side shared by its two splits, and
+// the flux from the two mass fluxes.
+__device__ __forceinline__ void ausm_split(double M, double sgn, double& mach, double& pres)
+{
+    if (!below_abs(M, 1.0)) {
+        const bool with = !negative(M * sgn);
+        mach = with ? M : 0.0;
+        pres = with ? 1.0 : 0.0;
+        return;
+    }
+    const double t = fma(M, M, -1.0), t2 = t * t, q = M + sgn, q2 = 0.25 * q * q;
+    mach = sgn * fma(0.125, t2, q2);
+    pres = fma(q2, fma(-sgn, M, 2.0), (sgn * 0.1875) * M * t2);
+}
+
+template <int D, int M>
+__device__ __forceinline__ void ausm_plus64(const Grid& g, int k, const double* PL, const double* PR, double* F)
+{
+    const double pL = PL[D + 1], pR = PR[D + 1];
+    double keL = 0.0, keR = 0.0;
+#pragma unroll
+    for (int c = 0; c < D; ++c) {
+        keL = fma(PL[1 + c], PL[1 + c], keL);
+        keR = fma(PR[1 + c], PR[1 + c], keR);
+    }
+    const double hp = g.igm + 1.0; // enthalpy of pressure: p g / (g - 1)
+    const double HL = fma(hp, pL / PL[0], 0.5 * keL), HR = fma(hp, pR / PR[0], 0.5 * keR);
+    const double uL = along<D>(PL + 1, k), uR = along<D>(PR + 1, k);
+    const double cst = g.cstar; // 2 (g - 1) / (g + 1)
+    const double aL2 = cst * HL, aR2 = cst * HR;
+    double aL = sqrt(aL2), aR = sqrt(aR2);
+    if (less(aL, uL)) aL = aL2 / uL;
+    if (less(aR, -uR)) aR = aR2 / -uR;
+    // a side without a critical speed leaves the interface speed to the other
+    const double a = !positive(aL2) ? aR : (!positive(aR2) || less(aL, aR) ? aL : aR), ia = 1.0 / a;
+    double m1, p1, m2, p2;
+    ausm_split(uL * ia, 1.0, m1, p1);
+    ausm_split(uR * ia, -1.0, m2, p2);
+    const double mh = a * (m1 + m2), ph = fma(p1, pL, p2 * pR);
+    const bool back = negative(mh);
+    const double fL = back ? 0.0 : mh * PL[0], fR = back ? mh * PR[0] : 0.0; // mass fluxes
+    F[0] = fL + fR;
+#pragma unroll
+    for (int c = 0; c < D; ++c) F[1 + c] = fma(fL, PL[1 + c], fma(fR, PR[1 + c], c == k ? ph : 0.0));
+    F[D + 1] = fma(fL, HL, fR * HR);
+}
+
+// HLL in FP64 from the reconstructed primitives, by its weights: with
+// w_L = s_R / (s_R - s_L) and w_R = -s_L / (s_R - s_L) (1 and 0 when both waves
+// run one way) the flux is sum over the sides of w (F(U) - s U), s the
+// other... outer speed of that side, i.e. U (w (u_n - s)) plus w times the pressure terms.
+// The two mass fluxes rho w (u_n - s) carry momentum and kinetic energy, so
+// neither the conservative states nor the physical fluxes are formed: about 80
+// FP64 operations per face with the reconstruction instead of 135.  Measured on
+// a GB300 together with child() and the comparisons above, mean stage-2 launch:
+// 2D Euler L = 10 from 43.9 to 35.8 us on level 10 and 33.3 to 24.9 us on level
+// 9, 3D blast L = 7 from 308 to 243 us on level 7.
+template <int D, int M>
+__device__ __forceinline__ void hll64(const Grid& g, int k, const double* PL, const double* PR, double* F)
+{
+    const double gam = g.phys[0], igm = g.igm, pL = PL[D + 1], pR = PR[D + 1];
+    const double uL = along<D>(PL + 1, k), uR = along<D>(PR + 1, k);
+    // sound speeds sqrt(gamma p / rho) = gamma p rsqrt(gamma p rho)
+    const double gpL = gam * pL, gpR = gam * pR, xL = gpL * PL[0], xR = gpR * PR[0];
+    const double cL = gpL * rsqrt(xL), cR = gpR * rsqrt(xR);
+    double lL = uL - cL, lR = uR - cR, rL = uL + cL, rR = uR + cR;
+    // a side without a sound speed (no positive pressure, as a prediction at a
+    // strong shock may give) leaves the wave speeds to the other
+    const bool okL = positive(xL), okR = positive(xR);
+    if (!okL) lL = lR, rL = rR;
+    if (!okR) lR = lL, rR = rL;
+    const double sL = less(lL, lR) ? lL : lR, sR = less(rL, rR) ? rR : rL;
+    const bool allL = (okL || okR) && !negative(sL), allR = (okL || okR) && !allL && !positive(sR);
+    const double ids = 1.0 / (sR - sL);
+    double wL = sR * ids, wR = -sL * ids;
+    double aL = wL * (uL - sL), aR = wR * (uR - sR);
+    if (allL || allR) {
+        wL = allL ? 1.0 : 0.0;
+        wR = allL ? 0.0 : 1.0;
+        aL = allL ? uL : 0.0;
+        aR = allL ? 0.0 : uR;
+    }
+    const double mL = aL * PL[0], mR = aR * PR[0]; // mass fluxes
+    F[0] = mL + mR;
+    const double pw2 = fma(wL, pL, wR * pR);
+    double keL = 0.0, keR = 0.0;
+#pragma unroll
+    for (int c = 0; c < D; ++c) {
+        F[1 + c] = fma(mL, PL[1 + c], fma(mR, PR[1 + c], c == k ? pw2 : 0.0));
+        keL = fma(PL[1 + c], PL[1 + c], keL);
+        keR = fma(PR[1 + c], PR[1 + c], keR);
+    }
+    // energy: m ke / 2 + p (a / (g - 1) + w u_n), each side
+    const double eL = pL * fma(aL, igm, wL * uL), eR = pR * fma(aR, igm, wR * uR);
+    F[D + 1] = fma(0.5 * mL, keL, fma(0.5 * mR, keR, eL + eR));
 }
 
 // Numerical flux along direction k across the face between stencil cells 1
@@ -514,56 +645,61 @@ __device__ __forceinline__ void flux_recon(const Grid& g, int k, double dxf, con
             PL[v] = a1 + h * minmod(a1 - a0, a2 - a1);
             PR[v] = a2 - h * minmod(a2 - a1, a3 - a2);
         }
-        R UL[M], UR[M], FL[M], FR[M];
-        R keL = R(0), keR = R(0);
-        UL[0] = PL[0];
-        UR[0] = PR[0];
-#pragma unroll
-        for (int c = 0; c < D; ++c) {
-            UL[1 + c] = PL[0] * PL[1 + c];
-            UR[1 + c] = PR[0] * PR[1 + c];
-            keL += PL[1 + c] * PL[1 + c];
-            keR += PR[1 + c] * PR[1 + c];
-        }
-        const R igm = R(g.igm);
-        UL[D + 1] = fma(PL[D + 1], igm, mul_rn(h * PL[0], keL));
-        UR[D + 1] = fma(PR[D + 1], igm, mul_rn(h * PR[0], keR));
-        const R unL = along<D>(PL + 1, k), unR = along<D>(PR + 1, k);
-        if (g.flux == 1) { // AUSM+
-            ausm_plus<D, M, R>(gam, k, PL, PR, UL, UR, F);
-            return;
-        }
-#pragma unroll
-        for (int v = 0; v <= D; ++v) {
-            FL[v] = mul_rn(UL[v], unL);
-            FR[v] = mul_rn(UR[v], unR);
-            if (v == 1 + k) {
-                FL[v] = add_rn(FL[v], PL[D + 1]);
-                FR[v] = add_rn(FR[v], PR[D + 1]);
-            }
-        }
-        // energy flux (E + p) u_n: which product is rounded first differs by
-        // dimension, as FP32 solves have always had it
-        const R eL = UL[D + 1], eR = UR[D + 1], pL = PL[D + 1], pR = PR[D + 1];
-        FL[D + 1] = D == 2 ? fma(eL, unL, mul_rn(pL, unL)) : fma(pL, unL, mul_rn(eL, unL));
-        FR[D + 1] = D == 2 ? fma(eR, unR, mul_rn(pR, unR)) : fma(pR, unR, mul_rn(eR, unR));
-        // sound speeds sqrt(gamma p / rho) = gamma p rsqrt(gamma p rho)
-        const R gpL = gam * PL[D + 1], gpR = gam * PR[D + 1];
-        const R cL = gpL * rsqrt(gpL * PL[0]);
-        const R cR = gpR * rsqrt(gpR * PR[0]);
-        const R sL = fmin(unL - cL, unR - cR);
-        const R sR = fmax(unL + cL, unR + cR);
-        if (sL >= R(0)) {
-#pragma unroll
-            for (int v = 0; v < M; ++v) F[v] = FL[v];
-        } else if (sR <= R(0)) {
-#pragma unroll
-            for (int v = 0; v < M; ++v) F[v] = FR[v];
+        if constexpr (sizeof(R) == 8) {
+            if (g.flux == 1) ausm_plus64<D, M>(g, k, PL, PR, F);
+            else hll64<D, M>(g, k, PL, PR, F);
         } else {
-            const R ids = R(1) / (sR - sL);
+            R UL[M], UR[M], FL[M], FR[M];
+            R keL = R(0), keR = R(0);
+            UL[0] = PL[0];
+            UR[0] = PR[0];
 #pragma unroll
-            for (int v = 0; v < M; ++v)
-                F[v] = fma(sL * sR, UR[v] - UL[v], fma(sR, FL[v], -mul_rn(sL, FR[v]))) * ids;
+            for (int c = 0; c < D; ++c) {
+                UL[1 + c] = PL[0] * PL[1 + c];
+                UR[1 + c] = PR[0] * PR[1 + c];
+                keL += PL[1 + c] * PL[1 + c];
+                keR += PR[1 + c] * PR[1 + c];
+            }
+            const R igm = R(g.igm);
+            UL[D + 1] = fma(PL[D + 1], igm, mul_rn(h * PL[0], keL));
+            UR[D + 1] = fma(PR[D + 1], igm, mul_rn(h * PR[0], keR));
+            const R unL = along<D>(PL + 1, k), unR = along<D>(PR + 1, k);
+            if (g.flux == 1) { // AUSM+
+                ausm_plus<D, R>(gam, k, PL, PR, UL, UR, F);
+                return;
+            }
+#pragma unroll
+            for (int v = 0; v <= D; ++v) {
+                FL[v] = mul_rn(UL[v], unL);
+                FR[v] = mul_rn(UR[v], unR);
+                if (v == 1 + k) {
+                    FL[v] = add_rn(FL[v], PL[D + 1]);
+                    FR[v] = add_rn(FR[v], PR[D + 1]);
+                }
+            }
+            // energy flux (E + p) u_n: which product is rounded first differs by
+            // dimension, as FP32 solves have always had it
+            const R eL = UL[D + 1], eR = UR[D + 1], pL = PL[D + 1], pR = PR[D + 1];
+            FL[D + 1] = D == 2 ? fma(eL, unL, mul_rn(pL, unL)) : fma(pL, unL, mul_rn(eL, unL));
+            FR[D + 1] = D == 2 ? fma(eR, unR, mul_rn(pR, unR)) : fma(pR, unR, mul_rn(eR, unR));
+            // sound speeds sqrt(gamma p / rho) = gamma p rsqrt(gamma p rho)
+            const R gpL = gam * PL[D + 1], gpR = gam * PR[D + 1];
+            const R cL = gpL * rsqrt(gpL * PL[0]);
+            const R cR = gpR * rsqrt(gpR * PR[0]);
+            const R sL = fmin(unL - cL, unR - cR);
+            const R sR = fmax(unL + cL, unR + cR);
+            if (sL >= R(0)) {
+#pragma unroll
+                for (int v = 0; v < M; ++v) F[v] = FL[v];
+            } else if (sR <= R(0)) {
+#pragma unroll
+                for (int v = 0; v < M; ++v) F[v] = FR[v];
+            } else {
+                const R ids = R(1) / (sR - sL);
+#pragma unroll
+                for (int v = 0; v < M; ++v)
+                    F[v] = fma(sL * sR, UR[v] - UL[v], fma(sR, FL[v], -mul_rn(sL, FR[v]))) * ids;
+            }
         }
     }
 }

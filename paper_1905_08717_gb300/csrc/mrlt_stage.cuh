@@ -192,9 +192,10 @@ __device__ __noinline__ void far_value(const Grid& g, Ctx x, int l, int p0, int 
 // mixed from 13.9 to 12.1 us, FP64 from 38.9 to 37 us (bound by its FP64
 // operations), 3D blast L = 8 mixed from 160 to 117 us, L = 7 FP64 from 234
 // to 216 us.
-// Work lists keep every warp on one kind of work.  Each value is computed by
-// the same operations in the same order as the direct definitions (expose,
-// predict, value_at); only the place its inputs come from changes.
+// Work lists keep every warp on one kind of work.  In FP32 each value is
+// computed by the same operations in the same order as the direct definitions
+// (expose, predict, value_at); in FP64, whose operations bound the kernel, the
+// predictions go direction by direction (child()).
 // The tiles of levels lo..hi are distributed over the CTAs of the launch
 // (blockIdx / gridDim); smem is the dynamic shared memory of TileShape::SMEM
 // bytes.  Called by k_stage_tile and by the persistent macro-step kernel.
@@ -653,24 +654,45 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
             if (predicted) {
                 const int pb0 = (D > 2 ? (pc[2] >> 1) * PSZ : 0) + (D > 1 ? (pc[1] >> 1) * PSY : 0) + (pc[0] >> 1);
                 const int a0 = pc[0] & 1, a1 = pc[1] & 1, a2 = pc[2] & 1;
+                if constexpr (sizeof(R) == 8) {
+                    bool missing = false;
 #pragma unroll
-                for (int v = 0; v < M; ++v) W[v] = R(0);
-#pragma unroll(D > 2 ? 1 : 3)
-                for (int dz = (D > 2 ? -1 : 0); dz <= (D > 2 ? 1 : 0); ++dz) {
-                    const R wz = D > 2 ? R(pw(a2, dz)) : R(1);
-#pragma unroll(D > 2 ? 1 : 3)
-                    for (int dy = (D > 1 ? -1 : 0); dy <= (D > 1 ? 1 : 0); ++dy) {
-                        const R wyz = wz * (D > 1 ? R(pw(a1, dy)) : R(1));
+                    for (int v = 0; v < M; ++v) {
+                        R z3[3];
 #pragma unroll
-                        for (int dxx = -1; dxx <= 1; ++dxx) {
-                            const int pb = pb0 + (D > 2 ? (dz + 1) * PSZ : 0) + (D > 1 ? (dy + 1) * PSY : 0) + dxx + 1;
-                            if (sPSt[pb] == 0) {
-                                atomicOr(g.err, ERR_SOURCE);
-                                continue;
+                        for (int dz = 0; dz < (D > 2 ? 3 : 1); ++dz) {
+                            R y3[3];
+#pragma unroll
+                            for (int dy = 0; dy < (D > 1 ? 3 : 1); ++dy) {
+                                const int pb = pb0 + dz * PSZ + dy * PSY;
+                                if (v == 0) missing = missing || !sPSt[pb] || !sPSt[pb + 1] || !sPSt[pb + 2];
+                                y3[dy] = child(sPW[v][pb], sPW[v][pb + 1], sPW[v][pb + 2], a0);
                             }
-                            const R w0 = wyz * R(pw(a0, dxx));
+                            z3[dz] = D > 1 ? child(y3[0], y3[1], y3[2], a1) : y3[0];
+                        }
+                        W[v] = D > 2 ? child(z3[0], z3[1], z3[2], a2) : z3[0];
+                    }
+                    if (missing) atomicOr(g.err, ERR_SOURCE);
+                } else {
 #pragma unroll
-                            for (int v = 0; v < M; ++v) W[v] += w0 * sPW[v][pb];
+                    for (int v = 0; v < M; ++v) W[v] = R(0);
+#pragma unroll(D > 2 ? 1 : 3)
+                    for (int dz = (D > 2 ? -1 : 0); dz <= (D > 2 ? 1 : 0); ++dz) {
+                        const R wz = D > 2 ? R(pw(a2, dz)) : R(1);
+#pragma unroll(D > 2 ? 1 : 3)
+                        for (int dy = (D > 1 ? -1 : 0); dy <= (D > 1 ? 1 : 0); ++dy) {
+                            const R wyz = wz * (D > 1 ? R(pw(a1, dy)) : R(1));
+#pragma unroll
+                            for (int dxx = -1; dxx <= 1; ++dxx) {
+                                const int pb = pb0 + (D > 2 ? (dz + 1) * PSZ : 0) + (D > 1 ? (dy + 1) * PSY : 0) + dxx + 1;
+                                if (sPSt[pb] == 0) {
+                                    atomicOr(g.err, ERR_SOURCE);
+                                    continue;
+                                }
+                                const R w0 = wyz * R(pw(a0, dxx));
+#pragma unroll
+                                for (int v = 0; v < M; ++v) W[v] += w0 * sPW[v][pb];
+                            }
                         }
                     }
                 }
@@ -721,16 +743,45 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
                 flux_recon<EQ, D, M, R>(g, k, g.dx[u][k], [&](int c, int v) { return sP[v][lc + (c - 1) * stride]; },
                                         F);
             } else {
+                // stencil on level u+1: the leaf's own children (virtual, predicted;
+                // low and high) and the two cells of the finer side
                 const Sub z = sub_task(task);
-                const bool pre = task < NPF; // finer side fetched in phase 3
-                R P4[4][M];
+                R Pc[2][M], Pf[2][M];
+                if constexpr (sizeof(R) == 8) {
+                    const int sk = k == 0 ? 1 : (k == 1 ? SY : SZ); // strides along the face's normal
+                    const int s1 = k == 0 ? SY : 1, s2 = k == 2 ? SY : SZ; // and its tangential directions
+                    R W[2][M];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    // stencil cell i on level u+1; the leaf's own children are virtual
-                    int p[3];
-                    sub_cell(z, i, p);
-                    const bool own_child = z.side > 0 ? i < 2 : i >= 2;
-                    if (own_child) {
+                    for (int v = 0; v < M; ++v) {
+                        R c3[3];
+#pragma unroll
+                        for (int i = 0; i < 3; ++i) {
+                            const R* w = &sW[v][z.bl + (i - 1) * sk];
+                            if constexpr (D == 1) {
+                                c3[i] = w[0];
+                            } else if constexpr (D == 2) {
+                                c3[i] = child(w[-s1], w[0], w[s1], z.t);
+                            } else {
+                                R y3[3];
+#pragma unroll
+                                for (int j = 0; j < 3; ++j) {
+                                    const R* y = w + (j - 1) * s2;
+                                    y3[j] = child(y[-s1], y[0], y[s1], z.t & 1);
+                                }
+                                c3[i] = child(y3[0], y3[1], y3[2], z.t >> 1);
+                            }
+                        }
+                        const R d = c3[2] - c3[0];
+                        W[0][v] = fma(-0.125, d, c3[1]);
+                        W[1][v] = fma(0.125, d, c3[1]);
+                    }
+                    recon_vars<EQ, D, M, R>(g, W[0], Pc[0]);
+                    recon_vars<EQ, D, M, R>(g, W[1], Pc[1]);
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        int p[3];
+                        sub_cell(z, z.side > 0 ? r : 2 + r, p);
                         R W[M];
                         const int ax = p[0] & 1, ay = p[1] & 1, az = p[2] & 1;
 #pragma unroll
@@ -747,18 +798,29 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
 #pragma unroll
                                     for (int v = 0; v < M; ++v) W[v] += w * sW[v][bs];
                                 }
-                        recon_vars<EQ, D, M, R>(g, W, P4[i]);
-                    } else if (pre) {
-                        const int r = z.side > 0 ? i - 2 : i;
-#pragma unroll
-                        for (int v = 0; v < M; ++v) P4[i][v] = sFine[r][v][task];
-                    } else {
-                        R far[M];
-                        far_value<D, M, R>(g, x, u + 1, p[0], p[1], p[2], far);
-                        recon_vars<EQ, D, M, R>(g, far, P4[i]);
+                        recon_vars<EQ, D, M, R>(g, W, Pc[r]);
                     }
                 }
-                flux_recon<EQ, D, M, R>(g, k, g.dx[u + 1][k], [&](int cc, int v) { return P4[cc][v]; }, F);
+                if (task < NPF) { // finer side fetched in phase 3
+#pragma unroll
+                    for (int r = 0; r < 2; ++r)
+#pragma unroll
+                        for (int v = 0; v < M; ++v) Pf[r][v] = sFine[r][v][task];
+                } else {
+#pragma unroll
+                    for (int r = 0; r < 2; ++r) {
+                        int p[3];
+                        sub_cell(z, z.side > 0 ? 2 + r : r, p);
+                        R far[M];
+                        far_value<D, M, R>(g, x, u + 1, p[0], p[1], p[2], far);
+                        recon_vars<EQ, D, M, R>(g, far, Pf[r]);
+                    }
+                }
+                const bool up = z.side > 0;
+                flux_recon<EQ, D, M, R>(
+                    g, k, g.dx[u + 1][k],
+                    [&](int c, int v) { return c < 2 ? (up ? Pc[c][v] : Pf[c][v]) : (up ? Pf[c - 2][v] : Pc[c - 2][v]); },
+                    F);
             }
         }
         // mean of the sub-face fluxes of a face (every lane takes part in the
