@@ -103,8 +103,11 @@ struct TileShape {
     // the parent block, reconstruction variables, face fluxes and the
     // prefetched finer-side variables
     static constexpr size_t SMEM = sizeof(R) * M * (2 * NBP + PB + NF + 2 * NPF);
-    // CTAs per SM that the registers are shared out for
-    static constexpr int PERSM = D == 1 ? 8 : (D == 2 ? (sizeof(R) == 4 ? 4 : 3) : 2);
+    // CTAs per SM that the registers are shared out for.  Measured on a GB300,
+    // solves of the benchmark cases: 2D FP32 4 / 5 / 6 per SM 99.3 / 97.1 / 97.4
+    // ms, 3D FP32 2 / 3 / 4 24.6 / 22.7 / 22.8 ms; 2D FP64 2 / 3 / 4 / 5 240 /
+    // 221.5 / 221.7 / 222.8 ms, 3D FP64 1 / 2 48.2 / 43.3 ms (bound by FP64 issue).
+    static constexpr int PERSM = D == 1 ? 8 : (D == 2 ? (sizeof(R) == 4 ? 5 : 3) : (sizeof(R) == 4 ? 3 : 2));
 };
 
 // Value, as the level-u stencil sees it at stage x.s (the rel = +1 rows of
