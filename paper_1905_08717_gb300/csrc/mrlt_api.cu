@@ -61,12 +61,15 @@ struct mr_solver {
     double prof_level_ms[LMAX + 1] = {};
     long long prof_launches = 0, prof_all0 = 0;
     unsigned long long work0[(LMAX + 1) * 4] = {};
-    // one macro step (2^{L-min} fine iterations) captured as a CUDA graph and
-    // replayed on `stream`; captured on an internal stream because the legacy
-    // default stream cannot be captured
+    // the pieces of a macro step captured as CUDA graphs and replayed on
+    // `stream` (see run_macro); captured on an internal stream because the
+    // legacy default stream cannot be captured
     cudaStream_t cap_stream = nullptr;
-    cudaGraphExec_t macro_exec = nullptr;
-    long long macro_launches = 0, macro_stage_launches = 0;
+    struct Piece {
+        cudaGraphExec_t exec = nullptr;
+        long long launches = 0, stage_launches = 0;
+    };
+    Piece first, inner, lead[LMAX + 1];
     bool graph_off = false; // capture failed once, or disabled by the caller
     // batched use: the macro-step finiteness check copies the device error
     // bits here (pinned host memory) instead of synchronising
@@ -262,6 +265,7 @@ mr_status alloc_nodes(mr_solver* h, Grid& g, long long cap, std::vector<void*>& 
 }
 
 void drop_graphs(mr_solver* h);
+bool captured(const mr_solver* h) { return h->first.exec || h->inner.exec || h->head_exec; }
 
 void free_allocs(mr_solver* h, std::vector<void*>& v)
 {
@@ -286,7 +290,7 @@ mr_status set_capacity(mr_solver* h, long long newcap, bool keep)
         for (int l = g.lb; l <= g.L; ++l) used += cnt[l] + cnt[LMAX + 1 + l];
         if (used + 1 > newcap) newcap = used + 1;
     }
-    if (h->macro_exec || h->head_exec) { // captured with the old arrays
+    if (captured(h)) { // with the old arrays
         MR_CK(cudaStreamSynchronize(h->stream));
         drop_graphs(h);
     }
@@ -442,8 +446,13 @@ mr_status run_iters(mr_solver* h, double dt, long long n);
 
 void drop_graphs(mr_solver* h)
 {
-    if (h->macro_exec) cudaGraphExecDestroy(h->macro_exec);
-    h->macro_exec = nullptr;
+    auto drop = [](mr_solver::Piece& x) {
+        if (x.exec) cudaGraphExecDestroy(x.exec);
+        x = mr_solver::Piece();
+    };
+    drop(h->first);
+    drop(h->inner);
+    for (auto& x : h->lead) drop(x);
     if (h->head_exec) cudaGraphExecDestroy(h->head_exec);
     h->head_exec = nullptr;
 }
@@ -544,7 +553,7 @@ mr_status sync_check(mr_solver* h)
 // part 1: details, thresholds and closure (the new tree in the flags); part
 // 2: the tree installed (slots released and taken), lists, projections; 0:
 // both.  A caller may check the node capacity between the parts.
-mr_status adapt(mr_solver* h, int la, int part = 0, long long it = 0)
+mr_status adapt(mr_solver* h, int la, int part = 0)
 {
     Grid& g = h->K.g;
     if (la >= g.L) return MR_OK;
@@ -554,7 +563,7 @@ mr_status adapt(mr_solver* h, int la, int part = 0, long long it = 0)
             h->K.scale();
         }
         // the flags are zero here: every remesh's compaction clears those it set
-        h->K.mark_refinements(la, part == 0 && can_halt(h) ? it : -1);
+        h->K.mark_refinements(la, part == 0 && can_halt(h));
     }
     if (part != 1) {
         h->K.apply_tree(la);
@@ -566,17 +575,18 @@ mr_status adapt(mr_solver* h, int la, int part = 0, long long it = 0)
 
 // one iteration n (0-based in the macro step) of Alg. 3
 // part 1 ends inside the adaptation, before the new tree is installed;
-// part 2 continues from there (see adapt); 0: the whole iteration
-mr_status lt_iteration(mr_solver* h, long long n, long long nit, int part = 0)
+// part 2 continues from there (see adapt); 0: the whole iteration but for the
+// reflux at its end (end_reflux)
+mr_status lt_iteration(mr_solver* h, long long n, int part = 0)
 {
     Grid& g = h->K.g;
     const int L = g.L, lb = g.lb, lmin = level_min(h, n);
     if (part != 2) {
-        h->K.leaf_copy(lmin, L, F_QE, F_Q0);
+        h->K.leaf_copy(lmin, L, F_QE, F_Q0, n > 0);
         h->K.project_up(L - 1, lmin, PM_Q0);
     }
     if (h->cfg.adapt_mode == MR_ADAPT_EVERY || (h->cfg.adapt_mode == MR_ADAPT_MACRO && n == 0))
-        MR_TRY(adapt(h, lmin, part, n));
+        MR_TRY(adapt(h, lmin, part));
     if (part == 1) return MR_OK;
     if (lmin > lb) h->K.project(lmin - 1, PM_MID);
     stage(h, lmin, L, 1, lmin); // first stage: all active levels at once
@@ -592,11 +602,16 @@ mr_status lt_iteration(mr_solver* h, long long n, long long nit, int part = 0)
             stage(h, l, l, 3, lmin);
         }
     }
-    if (h->reg) {
-        const int lc = (n + 1 == nit) ? lb : level_min(h, n + 1);
-        if (lc < L) h->K.reflux(lc, L - 1);
-    }
     return MR_OK;
+}
+
+// the reflux of the levels whose step ends before iteration n (nit: the end
+// of the macro step)
+void end_reflux(mr_solver* h, long long n, long long nit)
+{
+    if (!h->reg) return;
+    const int lc = n == nit ? h->K.g.lb : level_min(h, n);
+    if (lc < h->K.g.L) h->K.reflux(lc, h->K.g.L - 1);
 }
 
 // global time step MR (MR/RK2, MR/RK3)
@@ -605,11 +620,11 @@ mr_status gts_iteration(mr_solver* h, long long n, int part = 0)
     Grid& g = h->K.g;
     const int L = g.L, lb = g.lb;
     if (part != 2) {
-        h->K.leaf_copy(lb, L, F_QE, F_Q0);
+        h->K.leaf_copy(lb, L, F_QE, F_Q0, n > 0);
         h->K.project_up(L - 1, lb, PM_Q0);
     }
     if (h->cfg.adapt_mode == MR_ADAPT_EVERY || (h->cfg.adapt_mode == MR_ADAPT_MACRO && n == 0))
-        MR_TRY(adapt(h, lb, part, n));
+        MR_TRY(adapt(h, lb, part));
     if (part == 1) return MR_OK;
     stage(h, lb, L, 1, lb); // every level at the same instant: one launch per stage
     h->K.project_up(L - 1, lb, PM_Q1);
@@ -631,9 +646,17 @@ mr_status finite_check(mr_solver* h)
     return sync_check(h);
 }
 
+// iteration n without the reflux at its end
+mr_status open_iteration(mr_solver* h, long long n, int part = 0)
+{
+    return h->K.g.gts ? gts_iteration(h, n, part) : lt_iteration(h, n, part);
+}
+
 mr_status iteration(mr_solver* h, long long n, long long nit, int part = 0)
 {
-    return h->K.g.gts ? gts_iteration(h, n, part) : lt_iteration(h, n, nit, part);
+    MR_TRY(open_iteration(h, n, part));
+    if (part != 1) end_reflux(h, n + 1, nit);
+    return MR_OK;
 }
 
 // the part of iteration n that a macro step runs after its head (see the
@@ -642,8 +665,9 @@ int part_of(const mr_solver* h, long long n) { return n == 0 && split_head(h) ? 
 
 // Capture what `body` enqueues as a CUDA graph (stream capture on the
 // internal stream).  Every launch of a macro step is fixed by the layout,
-// the level schedule l_min(n) and the configuration; the fine step is read
-// from g.dtp, so one graph serves every macro step.  Returns false (and
+// the level schedule l_min(n) and the configuration; the fine step and the
+// iteration's number are read from device memory, so the graphs serve every
+// macro step.  Returns false (and
 // leaves nothing captured) when capture is not possible; the caller then
 // launches directly.
 template <class Body>
@@ -676,20 +700,62 @@ bool capture(mr_solver* h, Body body, cudaGraphExec_t* exec, long long* launches
     return ok;
 }
 
-// fine iterations [n0, n0 + cnt) of a macro step (iteration 0 from its head on)
-bool capture_iters(mr_solver* h, long long n0, long long cnt, long long nit, cudaGraphExec_t* exec,
-                   long long* launches, long long* stage_launches)
+// A macro step in pieces.  Iteration n is fixed by l_min(n), and that repeats:
+// between two multiples of a block length B = 2^b every block of the macro step
+// runs the same iterations 1..B-1, and the iteration on a multiple of B (with
+// the reflux that ends the step before it) depends only on its l_min.  So the
+// graphs captured are `first` (iteration 0 after its head), `inner` (iterations
+// 1..B-1) and `lead[l]` (the reflux down to level l, then an iteration with
+// l_min = l): B + L - lb - b iterations instead of all 2^{L-lb}, 19 against 128
+// for 2D Euler L = 10.  Capture and instantiation take about 3 us per launch on
+// the host of a GB300, and every resize of the node arrays repeats them: a 1D
+// Burgers solve of two macro steps at L = 10, made from nothing, takes 28.4 ms
+// against 39.8 ms with its macro step of 256 iterations captured whole, and a
+// batch of 24 reaction-diffusion problems 84 against 135 ms.
+constexpr long long kBlockIters = 16;
+
+long long block_iters(long long nit) { return nit < kBlockIters ? nit : kBlockIters; }
+
+bool capture_piece(mr_solver* h, mr_solver::Piece& x, long long reflux, long long n0, long long n1, long long nit)
 {
+    if (x.exec) return true;
     auto body = [&]() -> mr_status {
-        for (long long i = n0; i < n0 + cnt; ++i) MR_TRY(iteration(h, i, nit, part_of(h, i)));
+        if (reflux) end_reflux(h, reflux, nit);
+        for (long long n = n0; n < n1; ++n) {
+            MR_TRY(open_iteration(h, n, part_of(h, n)));
+            if (n + 1 < n1) end_reflux(h, n + 1, nit);
+        }
         return MR_OK;
     };
-    return capture(h, body, exec, launches, stage_launches);
+    return capture(h, body, &x.exec, &x.launches, &x.stage_launches);
 }
 
+// all pieces of a macro step; a failure leaves none
 bool capture_macro(mr_solver* h, long long nit)
 {
-    return capture_iters(h, 0, nit, nit, &h->macro_exec, &h->macro_launches, &h->macro_stage_launches);
+    const long long B = block_iters(nit);
+    bool ok = capture_piece(h, h->first, 0, 0, 1, nit);
+    if (B > 1) ok = ok && capture_piece(h, h->inner, 1, 1, B, nit);
+    for (long long n = B; n < nit && ok; n += B) ok = capture_piece(h, h->lead[level_min(h, n)], n, n, n + 1, nit);
+    if (!ok) drop_graphs(h);
+    return ok;
+}
+
+mr_status run_macro(mr_solver* h, long long nit)
+{
+    auto launch = [&](const mr_solver::Piece& x) -> mr_status {
+        MR_CK(cudaGraphLaunch(x.exec, h->stream));
+        h->K.n += x.launches;
+        h->stage_launches += x.stage_launches;
+        return MR_OK;
+    };
+    const long long B = block_iters(nit);
+    for (long long n = 0; n < nit; n += B) {
+        MR_TRY(launch(n == 0 ? h->first : h->lead[level_min(h, n)]));
+        if (B > 1) MR_TRY(launch(h->inner));
+    }
+    end_reflux(h, nit, nit);
+    return MR_OK;
 }
 
 // The head of the next macro step (iteration 0 up to the flags of the new
@@ -745,10 +811,6 @@ mr_status boundary_check(mr_solver* h)
     }
     return head_finish(h);
 }
-
-// Graphs are used for whole macro steps with profiling off, up to 1024 fine
-// iterations per macro step (larger schedules launch directly).
-constexpr long long kMaxGraphIters = 1024;
 
 // Profiling capacity of the macro-step kernel's phase stamps; a profiled run
 // launches at most kProfIters fine iterations per macro-step kernel.
@@ -875,15 +937,13 @@ mr_status run_iters(mr_solver* h, double dt, long long n)
             continue;
         }
         h->wmax_valid = false;
-        const bool can_graph = !h->prof && !h->graph_off && nit <= kMaxGraphIters;
+        const bool can_graph = !h->prof && !h->graph_off;
         if (can_graph && h->pos == 0 && left >= nit) { // a whole macro step
-            if (!h->macro_exec && !capture_macro(h, nit)) {
+            if (!capture_macro(h, nit)) {
                 h->graph_off = true; // launch directly from now on
                 continue;
             }
-            MR_CK(cudaGraphLaunch(h->macro_exec, h->stream));
-            h->K.n += h->macro_launches;
-            h->stage_launches += h->macro_stage_launches;
+            MR_TRY(run_macro(h, nit));
             advance(nit);
             continue;
         }
@@ -953,7 +1013,7 @@ mr_status init_state(mr_solver* h, const double* q0)
     MR_CK(cudaMemsetAsync(g.tflag, 0, h->tpad, h->stream));
     MR_CK(cudaMemsetAsync(g.counts, 0, 3 * (LMAX + 1) * sizeof(int), h->stream));
     MR_CK(cudaMemsetAsync(g.err, 0, sizeof(int), h->stream));
-    MR_CK(cudaMemsetAsync(g.room, 0, 4 * sizeof(int), h->stream));
+    MR_CK(cudaMemsetAsync(g.room, 0, 5 * sizeof(int), h->stream));
     MR_CK(cudaMemsetAsync(g.near, 0, sizeof(unsigned long long), h->stream));
     MR_CK(cudaMemsetAsync(g.updates, 0, sizeof(unsigned long long), h->stream));
     for (int l = g.lb; l <= g.L; ++l)
@@ -1046,7 +1106,7 @@ mr_status layout_alloc(mr_solver* h, const mr_config* cfg)
     A(dev_alloc(h, &g.tlist, (size_t)toff));
     A(dev_alloc(h, &g.scale_bits, MMAX));
     A(dev_alloc(h, &g.dtp, 1));
-    A(dev_alloc(h, &g.room, 4));
+    A(dev_alloc(h, &g.room, 5));
     A(dev_alloc(h, &g.err, 1));
     A(dev_alloc(h, &g.near, 1));
     A(dev_alloc(h, &g.wmax, 1));
@@ -1371,7 +1431,7 @@ mr_status mr_set_grid_cap(mr_solver* h, int ctas)
     if (h->K.g.gcap == ctas) return MR_OK;
     // a captured macro step holds the old launch shape: drop it once the
     // stream has passed it, and capture again at the next macro step
-    if (h->macro_exec || h->head_exec) {
+    if (captured(h)) {
         MR_CK(cudaStreamSynchronize(h->stream));
         drop_graphs(h);
     }

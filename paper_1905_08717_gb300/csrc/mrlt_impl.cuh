@@ -73,7 +73,8 @@ struct Grid {
     unsigned long long* updates;
     unsigned long long* work;       // [(LMAX+1) * 4]: leaf-stages per level and stage
     double* dtp;                    // fine step dt of the current macro step (device scalar)
-    int* room;                      // [0] refinement flags being counted, [1] halt: iteration + 1, [2] nodes needed
+    int* room;                      // [0] refinement flags being counted, [1] halt: iteration + 1, [2] nodes needed,
+                                    // [3] blocks that counted, [4] iteration of the macro step
     long long off[LMAX + 1];
     long long N[LMAX + 1];
     int n[LMAX + 1];

@@ -30,9 +30,10 @@ static inline int blocks_list(const Grid& g, int l)
 // runs one device body of mrlt_tree_dev.cuh over its own grid.
 // (T: the storage type of the fields, double or float)
 template <int M, class T>
-__global__ void k_leaf_copy(const __grid_constant__ Grid g, int lo, int hi, int from, int to)
+__global__ void k_leaf_copy(const __grid_constant__ Grid g, int lo, int hi, int from, int to, bool next)
 {
     MRLT_ENTER(g);
+    if (next && blockIdx.x == 0 && threadIdx.x == 0) ++g.room[4]; // the next iteration of the macro step begins
     dev_leaf_copy<M, T>(g, lo, hi, from, to);
 }
 
@@ -60,24 +61,24 @@ __global__ void k_detail(const __grid_constant__ Grid g, int lo, int hi)
 
 // Desired and admissible refinements in one pass: desire reads only the detail
 // bits, which the stores of the refinement bit keep.
-// it >= 0: this launch finalises the refinement flags (a remesh at level
+// check: this launch finalises the refinement flags (a remesh at level
 // la = L-1 has no closure), so it also checks that the new tree fits.
 template <int D>
-__global__ void k_mark(const __grid_constant__ Grid g, int lo, int hi, int la, long long it)
+__global__ void k_mark(const __grid_constant__ Grid g, int lo, int hi, int la, bool check)
 {
     MRLT_ENTER(g);
     dev_mark<D>(g, lo, hi, la);
-    if (it >= 0) room_decide(g, refined_here(g, la), la, it);
+    if (check) room_decide(g, refined_here(g, la), la);
 }
 
-// it >= 0: the last closure (level l-1 = la), which also checks that the new
+// check: the last closure (level l-1 = la), which also checks that the new
 // tree fits; its threads read back the level-la flags they wrote themselves
 template <int D>
-__global__ void k_close(const __grid_constant__ Grid g, int l, long long it)
+__global__ void k_close(const __grid_constant__ Grid g, int l, bool check)
 {
     MRLT_ENTER(g);
     dev_close<D>(g, l);
-    if (it >= 0) room_decide(g, refined_here(g, l - 1), l - 1, it);
+    if (check) room_decide(g, refined_here(g, l - 1), l - 1);
 }
 
 template <int D, int M, class T>
@@ -304,25 +305,28 @@ void Launcher::project_up(int hi, int lo, int mode)
 }
 
 template <int D, int M>
-static void leaf_copy_dm(Launcher& L, int lo, int hi, int from, int to)
+static void leaf_copy_dm(Launcher& L, int lo, int hi, int from, int to, bool next)
 {
-    MRLT_T_LAUNCH(L, blocks_list(L.g, hi), (L.g, lo, hi, from, to), k_leaf_copy<M);
+    MRLT_T_LAUNCH(L, blocks_list(L.g, hi), (L.g, lo, hi, from, to, next), k_leaf_copy<M);
     ++L.n;
 }
 
-void Launcher::leaf_copy(int lo, int hi, int from, int to) { MRLT_DM_DISPATCH(leaf_copy_dm, *this, lo, hi, from, to); }
+void Launcher::leaf_copy(int lo, int hi, int from, int to, bool next)
+{
+    MRLT_DM_DISPATCH(leaf_copy_dm, *this, lo, hi, from, to, next);
+}
 
 template <int D, int M>
-static void adapt_dm(Launcher& L, int la, long long it)
+static void adapt_dm(Launcher& L, int la, bool check)
 {
     const Grid& g = L.g;
     const int hi = g.L - 1; // levels whose nodes may own children
     if (g.prec) pdl_launch(k_detail<D, M, float>, blocks_list(g, hi), NTHREADS, 0, L.st, g, la, hi);
     else pdl_launch(k_detail<D, M, double>, blocks_list(g, hi), NTHREADS, 0, L.st, g, la, hi);
-    pdl_launch(k_mark<D>, blocks_step(g, hi), NTHREADS, 0, L.st, g, la, hi, la, la == hi ? it : -1LL);
+    pdl_launch(k_mark<D>, blocks_step(g, hi), NTHREADS, 0, L.st, g, la, hi, la, check && la == hi);
     L.n += 2;
     for (int l = g.L - 1; l > la; --l, ++L.n)
-        pdl_launch(k_close<D>, blocks_step(g, l - 1), NTHREADS, 0, L.st, g, l, l == la + 1 ? it : -1LL);
+        pdl_launch(k_close<D>, blocks_step(g, l - 1), NTHREADS, 0, L.st, g, l, check && l == la + 1);
 }
 
 
@@ -340,7 +344,7 @@ static void apply_dm(Launcher& L, int la)
     }
 }
 
-void Launcher::mark_refinements(int la, long long it) { MRLT_DM_DISPATCH(adapt_dm, *this, la, it); }
+void Launcher::mark_refinements(int la, bool check) { MRLT_DM_DISPATCH(adapt_dm, *this, la, check); }
 void Launcher::apply_tree(int la) { MRLT_DM_DISPATCH(apply_dm, *this, la); }
 
 void Launcher::compact(int lo, int hi)
@@ -370,7 +374,10 @@ __global__ void k_scale_init(Grid g)
 __global__ void k_set_dt(Grid g, double dt)
 {
     pdl_enter();
-    if (threadIdx.x == 0) *g.dtp = dt;
+    if (threadIdx.x == 0) {
+        *g.dtp = dt;
+        g.room[4] = 0; // iteration 0
+    }
 }
 
 // leaf values from (level, i, j, k) keys: q^n and the end value of each leaf

@@ -14,14 +14,15 @@ struct Launcher {
 
     void project(int l, int mode);
     void project_up(int hi, int lo, int mode); // levels hi..lo, fewer launches
-    void leaf_copy(int lo, int hi, int from, int to); // leaves of levels lo..hi
-    void mark_refinements(int la, long long it = -1); // it >= 0: check that the tree fits (halt)
+    // leaves of levels lo..hi; next: this begins the next iteration of the macro step
+    void leaf_copy(int lo, int hi, int from, int to, bool next = false);
+    void mark_refinements(int la, bool check = false); // check that the tree fits (halt)
     void apply_tree(int la);
     void compact(int lo, int hi);                      // leaf / node / tile lists of levels lo..hi
     void reflux(int lo, int hi);                       // coarse levels lo..hi
     void scale();                                      // running max |q_v| over all leaves
     void scale_init();                                 // running max |q_v| := 1e-14
-    void set_dt(double dt);                            // *g.dtp := dt
+    void set_dt(double dt);                            // *g.dtp := dt, iteration 0
     void set_leaves(const int* keys, const double* vals, long long count); // leaf q^n and end values
     void store_finest(const double* src); // finest-level q^n from double data [v][cell]
     void slots_full(long long ntot);      // every cell of every level a node (a new solver's tree)

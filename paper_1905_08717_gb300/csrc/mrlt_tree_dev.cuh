@@ -694,17 +694,18 @@ __device__ __forceinline__ void dev_close(const Grid& g, int l)
     }
 }
 
-// Does the tree flagged by a remesh at level la (fine iteration it) fit the
+// Does the tree flagged by a remesh at level la fit the
 // node arrays?  Each thread of the kernel that finalises the flags counted
 // `c` refined cells (the kernel's cells of levels la..L-1 in one flat
 // grid-stride range over them); the blocks add their counts into room[0].
 // The new tree has 2^d nodes above level la per refined cell, and the slots
 // it may take are the free ones plus those of the nodes above level la now
 // (the remesh releases them first).  The last block to finish (ticket
-// room[3]) decides: short of slots, the solver halts at this iteration,
-// room[1] = it + 1, room[2] = the nodes of the new tree (see halted()).
+// room[3]) decides: short of slots, the solver halts at this iteration (room[4],
+// counted on by its first kernel), room[1] = it + 1, room[2] = the nodes of
+// the new tree (see halted()).
 // Called by every thread of the block.
-__device__ __forceinline__ void room_decide(const Grid& g, int c, int la, long long it)
+__device__ __forceinline__ void room_decide(const Grid& g, int c, int la)
 {
     __shared__ int blk;
     if (threadIdx.x == 0) blk = 0;
@@ -727,7 +728,7 @@ __device__ __forceinline__ void room_decide(const Grid& g, int c, int la, long l
     }
     if (fresh > g.ftop[0] + above) {
         g.room[2] = (int)(below + fresh);
-        g.room[1] = (int)(it + 1);
+        g.room[1] = g.room[4] + 1;
     }
 }
 
