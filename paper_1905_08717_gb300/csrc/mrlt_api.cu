@@ -552,8 +552,9 @@ mr_status sync_check(mr_solver* h)
 // Algs. 1-2 restricted to levels >= la (full adaptation for la = min_level)
 // part 1: details, thresholds and closure (the new tree in the flags); part
 // 2: the tree installed (slots released and taken), lists, projections; 0:
-// both.  A caller may check the node capacity between the parts.
-mr_status adapt(mr_solver* h, int la, int part = 0)
+// both.  A caller may check the node capacity between the parts.  mid: the
+// mid-step level la - 1 is refreshed with the last sweep.
+mr_status adapt(mr_solver* h, int la, int part = 0, bool mid = false)
 {
     Grid& g = h->K.g;
     if (la >= g.L) return MR_OK;
@@ -568,7 +569,8 @@ mr_status adapt(mr_solver* h, int la, int part = 0)
     if (part != 1) {
         h->K.apply_tree(la);
         h->K.compact(la, g.L);
-        h->K.project_up(g.L - 1, la, PM_Q0);
+        if (mid) h->K.project_up(g.L - 1, la - 1, PM_Q0, PM_MID);
+        else h->K.project_up(g.L - 1, la, PM_Q0);
     }
     return MR_OK;
 }
@@ -581,24 +583,25 @@ mr_status lt_iteration(mr_solver* h, long long n, int part = 0)
 {
     Grid& g = h->K.g;
     const int L = g.L, lb = g.lb, lmin = level_min(h, n);
+    const bool remesh =
+        lmin < L && (h->cfg.adapt_mode == MR_ADAPT_EVERY || (h->cfg.adapt_mode == MR_ADAPT_MACRO && n == 0));
+    const bool mid = lmin > lb; // the mid-step level lmin - 1 is refreshed (Sec. 4.3)
     if (part != 2) {
-        h->K.leaf_copy(lmin, L, F_QE, F_Q0, n > 0);
-        h->K.project_up(L - 1, lmin, PM_Q0);
+        if (mid && !remesh) h->K.begin(lmin, n > 0, lmin - 1, PM_MID);
+        else h->K.begin(lmin, n > 0, lmin, PM_BEG);
     }
-    if (h->cfg.adapt_mode == MR_ADAPT_EVERY || (h->cfg.adapt_mode == MR_ADAPT_MACRO && n == 0))
-        MR_TRY(adapt(h, lmin, part));
+    if (remesh) MR_TRY(adapt(h, lmin, part, mid));
     if (part == 1) return MR_OK;
-    if (lmin > lb) h->K.project(lmin - 1, PM_MID);
     stage(h, lmin, L, 1, lmin); // first stage: all active levels at once
-    h->K.project_up(L - 1, lmin, PM_REF2);
+    h->K.project_up(L - 1, lmin, PM_REF2, -1, true);
     for (int l = L; l >= lmin; --l) {
-        if (l < L) h->K.project(l, PM_PRJ2);
+        if (l < L) h->K.project(l, PM_PRJ2, true);
         stage(h, l, l, 2, lmin);
     }
     if (g.rk == 3) {
-        h->K.project_up(L - 1, lmin, PM_REF3);
+        h->K.project_up(L - 1, lmin, PM_REF3, -1, true);
         for (int l = L; l >= lmin; --l) {
-            if (l < L) h->K.project(l, PM_PRJ3);
+            if (l < L) h->K.project(l, PM_PRJ3, true);
             stage(h, l, l, 3, lmin);
         }
     }
@@ -620,17 +623,16 @@ mr_status gts_iteration(mr_solver* h, long long n, int part = 0)
     Grid& g = h->K.g;
     const int L = g.L, lb = g.lb;
     if (part != 2) {
-        h->K.leaf_copy(lb, L, F_QE, F_Q0, n > 0);
-        h->K.project_up(L - 1, lb, PM_Q0);
+        h->K.begin(lb, n > 0, lb, PM_BEG);
     }
     if (h->cfg.adapt_mode == MR_ADAPT_EVERY || (h->cfg.adapt_mode == MR_ADAPT_MACRO && n == 0))
         MR_TRY(adapt(h, lb, part));
     if (part == 1) return MR_OK;
     stage(h, lb, L, 1, lb); // every level at the same instant: one launch per stage
-    h->K.project_up(L - 1, lb, PM_Q1);
+    h->K.project_up(L - 1, lb, PM_Q1, -1, true);
     stage(h, lb, L, 2, lb);
     if (g.rk == 3) {
-        h->K.project_up(L - 1, lb, PM_Q2);
+        h->K.project_up(L - 1, lb, PM_Q2, -1, true);
         stage(h, lb, L, 3, lb);
     }
     return MR_OK;
@@ -710,8 +712,7 @@ bool capture(mr_solver* h, Body body, cudaGraphExec_t* exec, long long* launches
 // for 2D Euler L = 10.  Capture and instantiation take about 3 us per launch on
 // the host of a GB300, and every resize of the node arrays repeats them: a 1D
 // Burgers solve of two macro steps at L = 10, made from nothing, takes 28.4 ms
-// against 39.8 ms with its macro step of 256 iterations captured whole, and a
-// batch of 24 reaction-diffusion problems 84 against 135 ms.
+// against 39.8 ms with its macro step of 256 iterations captured whole.
 constexpr long long kBlockIters = 16;
 
 long long block_iters(long long nit) { return nit < kBlockIters ? nit : kBlockIters; }
@@ -1014,6 +1015,7 @@ mr_status init_state(mr_solver* h, const double* q0)
     MR_CK(cudaMemsetAsync(g.counts, 0, 3 * (LMAX + 1) * sizeof(int), h->stream));
     MR_CK(cudaMemsetAsync(g.err, 0, sizeof(int), h->stream));
     MR_CK(cudaMemsetAsync(g.room, 0, 5 * sizeof(int), h->stream));
+    MR_CK(cudaMemsetAsync(g.tick, 0, 2 * sizeof(int), h->stream));
     MR_CK(cudaMemsetAsync(g.near, 0, sizeof(unsigned long long), h->stream));
     MR_CK(cudaMemsetAsync(g.updates, 0, sizeof(unsigned long long), h->stream));
     for (int l = g.lb; l <= g.L; ++l)
@@ -1106,6 +1108,7 @@ mr_status layout_alloc(mr_solver* h, const mr_config* cfg)
     A(dev_alloc(h, &g.tlist, (size_t)toff));
     A(dev_alloc(h, &g.scale_bits, MMAX));
     A(dev_alloc(h, &g.dtp, 1));
+    A(dev_alloc(h, &g.tick, 2));
     A(dev_alloc(h, &g.room, 5));
     A(dev_alloc(h, &g.err, 1));
     A(dev_alloc(h, &g.near, 1));

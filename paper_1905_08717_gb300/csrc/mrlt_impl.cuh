@@ -72,6 +72,7 @@ struct Grid {
     unsigned long long* wmax;
     unsigned long long* updates;
     unsigned long long* work;       // [(LMAX+1) * 4]: leaf-stages per level and stage
+    int* tick;                      // [2] tile tickets of stage launches, by parity of the stage
     double* dtp;                    // fine step dt of the current macro step (device scalar)
     int* room;                      // [0] refinement flags being counted, [1] halt: iteration + 1, [2] nodes needed,
                                     // [3] blocks that counted, [4] iteration of the macro step

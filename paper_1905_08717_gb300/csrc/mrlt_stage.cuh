@@ -199,14 +199,28 @@ __device__ __noinline__ void far_value(const Grid& g, Ctx x, int l, int p0, int 
 // computed by the same operations in the same order as the direct definitions
 // (expose, predict, value_at); in FP64, whose operations bound the kernel, the
 // predictions go direction by direction (child()).
-// The tiles of levels lo..hi are distributed over the CTAs of the launch
-// (blockIdx / gridDim); smem is the dynamic shared memory of TileShape::SMEM
-// bytes.  Called by k_stage_tile and by the persistent macro-step kernel.
-template <int EQ, int D, class R>
+// The tiles of levels lo..hi are distributed over the CTAs of the launch; smem
+// is the dynamic shared memory of TileShape::SMEM bytes.  Called by
+// k_stage_tile and by the persistent macro-step kernel.
+//
+// EARLY (k_stage_tile): phases 1 and 2 read nothing but the tree, and no
+// kernel that changes the tree comes directly before a stage launch.  So they
+// run before the wait for that kernel's results (pdl_enter): when this launch
+// starts, every CTA of its predecessor has itself waited for its own, so
+// whatever built the tree is complete.  The first tile's status trips, masks and
+// lookups thus overlap the predecessor.  CTAs that start early land on SMs
+// unevenly, so a launch with more tiles than CTAs hands out those after every
+// CTA's first by a counter, in the order the CTAs ask (tiles fixed to CTAs made
+// an early start 10% slower).  The CTA that takes the last ticket clears the
+// counter.  Two counters by the parity of the stage: the
+// launch before the last that uses the same one is complete when this one
+// starts.
+template <int EQ, int D, class R, bool EARLY>
 __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s, int lmin, double bstage, int reg,
                                             unsigned char* smem)
 {
-    const double dt = *g.dtp; // fine step of the macro step
+    const bool halt = halted(g); // with the loads below in one trip
+    const double dt = *g.dtp;    // fine step of the macro step
     using S = TileShape<EQ, D, R>;
     using Bits = typename Tile<D>::Bits;
     constexpr int M = S::M, TX = S::TX, TY = S::TY, TZ = S::TZ, NT = S::NT, H = S::H, NC = S::NC;
@@ -242,10 +256,18 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
     // in level order; one launch may cover several independent levels.
     int ntask = 0;
     for (int l = lo; l <= hi; ++l) ntask += g.counts[2 * (LMAX + 1) + l];
-    for (int task = blockIdx.x; task < ntask; task += gridDim.x) {
+    // the first tile of a one-level launch comes with the counts (its list has
+    // an entry for every tile of the level)
+    const bool one = lo == hi && (int)blockIdx.x < g.ntx[lo] * g.nty[lo] * g.ntz[lo];
+    const int tile0 = one ? g.tlist[g.toff[lo] + blockIdx.x] : 0;
+    if (halt) ntask = 0;
+    bool waited = !EARLY;
+    const bool handed = EARLY && ntask > (int)gridDim.x; // tiles beyond the first by tickets
+    __shared__ int sNext;
+    for (int task = blockIdx.x; task < ntask;) {
     int u = lo, at = task;
     for (int c; at >= (c = g.counts[2 * (LMAX + 1) + u]); ++u) at -= c;
-    const int tile = g.tlist[g.toff[u] + at];
+    const int tile = one && task == (int)blockIdx.x ? tile0 : g.tlist[g.toff[u] + at];
     const double dtl = g.gts ? dt : ldexp(dt, g.L - u); // Eq. 13 step of level u
     const double bw = dtl * bstage; // register weight dt_l b_s
     const int n = g.n[u];
@@ -301,6 +323,11 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
     if (tid < PBY * PBZ) sPar[tid] = 0;
     if (tid == 0) sWord[0][NW] = sWord[1][NW] = 0;
     __syncthreads();
+    if (handed && tid == 0) {
+        const int ticket = atomicAdd(&g.tick[s & 1], 1);
+        if (ticket == ntask - 1) g.tick[s & 1] = 0;
+        sNext = (int)gridDim.x + ticket;
+    }
 
     // 2. row masks.  row(k, by, bz): the leaves (k = 0) or internal nodes (1)
     // of a row of the block, empty past it; tile_row: the tile's leaves in it
@@ -557,6 +584,10 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
         }
     }
     __syncthreads();
+    if (!waited) { // from here on values are read
+        pdl_enter();
+        waited = true;
+    }
     const int nst = sCount[0], nvc = sCount[1], nlf = sCount[2];
 
     // 3. one trip: exposures of stored and parent cells and of the finer-side
@@ -895,16 +926,17 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
         rk_update<M, R>(g, sl, v, s, R(dtl), f, q0p, self);
     }
     __syncthreads(); // shared arrays are reused by the next tile
+    task = handed ? sNext : task + (int)gridDim.x;
     }
+    if (!waited) pdl_enter(); // no tile: the kernels after this one rely on its wait
 }
 
 template <int EQ, int D, class R>
 __global__ void __launch_bounds__(Tile<D>::THREADS, TileShape<EQ, D, R>::PERSM)
 k_stage_tile(const __grid_constant__ Grid g, int lo, int hi, int s, int lmin, double bstage, int reg)
 {
-    MRLT_ENTER(g);
     extern __shared__ __align__(16) unsigned char smem[];
-    stage_tiles<EQ, D, R>(g, lo, hi, s, lmin, bstage, reg, smem);
+    stage_tiles<EQ, D, R, true>(g, lo, hi, s, lmin, bstage, reg, smem);
 }
 
 static inline int grid_for(const Grid& g, int l)
@@ -916,9 +948,9 @@ static inline int grid_for(const Grid& g, int l)
 // One launch of the tiled stage kernel over the active tiles of levels lo..hi;
 // the persistent grid is the device's resident capacity for this instantiation
 // (occupancy API, once per device), capped by the tile count and by g.gcap
-// when that is set.  CTAs stride over the tile slots and every cell's update
-// and flux registers are written by one thread, so the result does not depend
-// on the grid size.
+// when that is set.  Every cell's update and flux registers are written by one
+// thread, so the result does not depend on the grid size or on which CTA
+// takes a tile.
 template <int EQ, int D, class R>
 static int stage_dispatch(const Grid& g, cudaStream_t st, int lo, int hi, int s, int lmin, double b, int reg)
 {
@@ -944,9 +976,9 @@ static int stage_dispatch(const Grid& g, cudaStream_t st, int lo, int hi, int s,
     long long grid = total < resident[dev] ? total : resident[dev];
     if (g.gcap > 0 && grid > g.gcap) grid = g.gcap;
     if (grid < 1) grid = 1;
-    // launched without a programmatic dependency: the persistent grid assigns
-    // tiles statically, so it must find the SMs free to be resident at once
-    k_stage_tile<EQ, D, R><<<(unsigned)grid, S::NT, S::SMEM, st>>>(g, lo, hi, s, lmin, b, reg);
+    if (pdl_launch(k_stage_tile<EQ, D, R>, dim3((unsigned)grid), dim3(S::NT), S::SMEM, st, g, lo, hi, s, lmin, b, reg) !=
+        cudaSuccess)
+        return -1;
     return 1;
 }
 

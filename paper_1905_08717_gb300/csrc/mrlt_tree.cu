@@ -27,36 +27,70 @@ static inline int blocks_list(const Grid& g, int l)
 
 // ------------------------------------------------------------ kernels
 // Each kernel waits for its predecessor (programmatic dependent launch) and
-// runs one device body of mrlt_tree_dev.cuh over its own grid.
+// runs one device body of mrlt_tree_dev.cuh over its own grid; kernels whose
+// predecessor leaves the tree alone look it up before they wait.  Most launches
+// are short chains of dependent trips, so that takes two or three of five trips
+// off them.  Measured on a GB300 with the stage kernel's early start, whole
+// solves: 1D Burgers L = 10 30.5 to 23.6 ms (made from nothing), 2D Burgers
+// L = 10 109.6 to 94.4 ms, 2D Euler L = 10 mixed 67.3 to 59.4 ms, global step
+// L = 9 64.6 to 60.6 ms, 3D blast L = 7 48.4 to 45.6 ms.
 // (T: the storage type of the fields, double or float)
 template <int M, class T>
-__global__ void k_leaf_copy(const __grid_constant__ Grid g, int lo, int hi, int from, int to, bool next)
+__global__ void k_leaf_copy(const __grid_constant__ Grid g, int lo, int hi, int from, int to)
 {
     MRLT_ENTER(g);
-    if (next && blockIdx.x == 0 && threadIdx.x == 0) ++g.room[4]; // the next iteration of the macro step begins
     dev_leaf_copy<M, T>(g, lo, hi, from, to);
 }
 
+// Up-sweep of levels hi..lo (one level: hi = lo); early as in kernel_list.
 template <int D, int M, class T>
-__global__ void k_project(const __grid_constant__ Grid g, int l, int mode)
+__global__ void k_project_up(const __grid_constant__ Grid g, int hi, int lo, int mode, int top, bool early)
 {
-    MRLT_ENTER(g);
-    dev_project<D, M, T>(g, l, mode);
+    if (!early) pdl_enter();
+    const int steps = up_steps(g, hi, lo);
+    for (int c = blockIdx.x; c < steps || early; c += gridDim.x) { // uniform across the CTA
+        const UpRefs<D> r = up_lookup<D>(g, hi, lo, c);
+        if (early) {
+            pdl_enter();
+            early = false;
+        }
+        if (halted(g)) return;
+        up_project<D, M, T>(g, r, hi - lo, mode, top);
+    }
 }
 
-// up-sweep of levels hi..lo in one launch (dev_project_up)
+// The beginning of an iteration: q^n := end value of the leaves of levels
+// lo..L and, beside it, the up-sweep of levels uhi..ulo (which reads leaf
+// children's end values; ulo with mode top): one launch where the copy and the
+// sweep were two.  The tree is looked up before the wait, as in kernel_list: an
+// iteration's predecessor never changes the tree.
 template <int D, int M, class T>
-__global__ void k_project_up(const __grid_constant__ Grid g, int hi, int lo, int mode)
+__global__ void k_begin(const __grid_constant__ Grid g, int lo, bool next, int uhi, int ulo, int top)
 {
-    MRLT_ENTER(g);
-    dev_project_up<D, M, T>(g, hi, lo, mode);
+    const int steps = uhi >= ulo ? up_steps(g, uhi, ulo) : 0;
+    UpRefs<D> r;
+    if (uhi >= ulo) r = up_lookup<D>(g, uhi, ulo, blockIdx.x);
+    kernel_list<0>(
+        g, lo, g.L, true, [&](int l, long long id) { return slot_of(g, l, id); },
+        [&](int sl) {
+            T q[M];
+            load_row<M, T>(nd<T>(g, F_QE, sl), q);
+            store_row<M, T>(nd<T>(g, F_Q0, sl), q);
+        });
+    if (halted(g)) return;
+    if (next && blockIdx.x == 0 && threadIdx.x == 0) ++g.room[4]; // the next iteration of the macro step
+    for (int c = blockIdx.x; c < steps; c += gridDim.x) { // uniform across the CTA
+        if (c != (int)blockIdx.x) r = up_lookup<D>(g, uhi, ulo, c);
+        up_project<D, M, T>(g, r, uhi - ulo, PM_BEG, top);
+    }
 }
 
 template <int D, int M, class T>
 __global__ void k_detail(const __grid_constant__ Grid g, int lo, int hi)
 {
-    MRLT_ENTER(g);
-    dev_detail<D, M, T>(g, lo, hi);
+    kernel_list<1>(
+        g, lo, hi, true, [&](int l, long long id) { return lookup_detail<D>(g, l, id); },
+        [&](const DetailRefs<D>& e) { detail_node<D, M, T>(g, e); });
 }
 
 // Desired and admissible refinements in one pass: desire reads only the detail
@@ -118,8 +152,9 @@ __global__ void k_cmp_scatter(const __grid_constant__ Grid g, LevelChunks lc, co
 template <int D, int M, class T>
 __global__ void k_reflux(const __grid_constant__ Grid g, int lo, int hi)
 {
-    MRLT_ENTER(g);
-    dev_reflux<D, M, T>(g, lo, hi);
+    kernel_list<0>(
+        g, lo, hi, true, [&](int l, long long id) { return lookup_reflux<D>(g, l, id); },
+        [&](const RefluxRefs<D>& e) { reflux_leaf<D, M, T>(g, e); });
 }
 
 // ------------------------------------------------------------ reductions
@@ -267,54 +302,59 @@ __global__ void k_uni_down(Grid g, int l, double* T, uint8_t* us)
     } while (0)
 #define MRLT_UNPACK(...) __VA_ARGS__
 
-template <int D, int M>
-static void project_dm(Launcher& L, int l, int mode)
-{
-    MRLT_T_LAUNCH(L, blocks_list(L.g, l), (L.g, l, mode), k_project<D, M);
-    ++L.n;
-}
-
-void Launcher::project(int l, int mode) { MRLT_DM_DISPATCH(project_dm, *this, l, mode); }
-
 // Up-sweep hi -> lo in groups of at most 6 / d + 1 levels per launch: a group
 // [glo, ghi] has 2^{d (ghi - glo)} <= 64 descendants per top node, so two top
-// nodes fit the NTHREADS = 128 threads of a CTA.
-template <int D, int M>
-static void project_up_dm(Launcher& L, int hi, int lo, int mode)
+// nodes fit the NTHREADS = 128 threads of a CTA.  Level lo takes mode `top`.
+static int up_blocks(const Grid& g, int ghi, int glo)
 {
-    constexpr int kDepth = 6 / D;
-    static_assert((1 << (D * kDepth)) * 2 <= NTHREADS, "two top nodes per CTA");
+    if (ghi <= glo) return blocks_list(g, glo);
+    const int tops = NTHREADS >> (g.d * (ghi - glo));
+    const long long b = (g.N[glo] + tops - 1) / tops;
+    return (int)(b > 1216 ? 1216 : b);
+}
+
+template <int D, int M>
+static void project_up_dm(Launcher& L, int hi, int lo, int mode, int top, bool early)
+{
+    static_assert((1 << (D * kUpDepth<D>)) * 2 <= NTHREADS, "two top nodes per CTA");
     for (int ghi = hi; ghi >= lo;) {
-        const int glo = ghi - kDepth > lo ? ghi - kDepth : lo;
-        if (glo == ghi) {
-            project_dm<D, M>(L, ghi, mode);
-        } else {
-            const int tops = NTHREADS >> (D * (ghi - glo));
-            long long b = (L.g.N[glo] + tops - 1) / tops;
-            if (b > 1216) b = 1216;
-            MRLT_T_LAUNCH(L, (int)b, (L.g, ghi, glo, mode), k_project_up<D, M);
-            ++L.n;
-        }
+        const int glo = ghi - kUpDepth<D> > lo ? ghi - kUpDepth<D> : lo;
+        MRLT_T_LAUNCH(L, up_blocks(L.g, ghi, glo), (L.g, ghi, glo, mode, glo == lo ? top : mode, early),
+                      k_project_up<D, M);
+        ++L.n;
         ghi = glo - 1;
+        early = true; // a sweep changes no tree
     }
 }
 
-void Launcher::project_up(int hi, int lo, int mode)
+void Launcher::project(int l, int mode, bool early) { MRLT_DM_DISPATCH(project_up_dm, *this, l, l, mode, mode, early); }
+
+void Launcher::project_up(int hi, int lo, int mode, int top, bool early)
 {
-    if (hi >= lo) MRLT_DM_DISPATCH(project_up_dm, *this, hi, lo, mode);
+    if (hi >= lo) MRLT_DM_DISPATCH(project_up_dm, *this, hi, lo, mode, top < 0 ? mode : top, early);
 }
 
 template <int D, int M>
-static void leaf_copy_dm(Launcher& L, int lo, int hi, int from, int to, bool next)
+static void begin_dm(Launcher& L, int lmin, bool next, int lo, int top)
 {
-    MRLT_T_LAUNCH(L, blocks_list(L.g, hi), (L.g, lo, hi, from, to, next), k_leaf_copy<M);
+    const Grid& g = L.g;
+    const int ghi = g.L - 1, glo = ghi - kUpDepth<D> > lo ? ghi - kUpDepth<D> : lo;
+    const int b0 = blocks_list(g, g.L), b1 = ghi >= lo ? up_blocks(g, ghi, glo) : 1;
+    MRLT_T_LAUNCH(L, b0 > b1 ? b0 : b1, (g, lmin, next, ghi, glo, glo == lo ? top : (int)PM_BEG), k_begin<D, M);
+    ++L.n;
+    if (glo > lo) project_up_dm<D, M>(L, glo - 1, lo, PM_BEG, top, true);
+}
+
+void Launcher::begin(int lmin, bool next, int lo, int top) { MRLT_DM_DISPATCH(begin_dm, *this, lmin, next, lo, top); }
+
+template <int D, int M>
+static void leaf_copy_dm(Launcher& L, int lo, int hi, int from, int to)
+{
+    MRLT_T_LAUNCH(L, blocks_list(L.g, hi), (L.g, lo, hi, from, to), k_leaf_copy<M);
     ++L.n;
 }
 
-void Launcher::leaf_copy(int lo, int hi, int from, int to, bool next)
-{
-    MRLT_DM_DISPATCH(leaf_copy_dm, *this, lo, hi, from, to, next);
-}
+void Launcher::leaf_copy(int lo, int hi, int from, int to) { MRLT_DM_DISPATCH(leaf_copy_dm, *this, lo, hi, from, to); }
 
 template <int D, int M>
 static void adapt_dm(Launcher& L, int la, bool check)

@@ -12,10 +12,14 @@ struct Launcher {
     int* bc = nullptr; // compaction scratch, 2 ints per block over all levels
     long long n = 0;   // kernel launches issued
 
-    void project(int l, int mode);
-    void project_up(int hi, int lo, int mode); // levels hi..lo, fewer launches
-    // leaves of levels lo..hi; next: this begins the next iteration of the macro step
-    void leaf_copy(int lo, int hi, int from, int to, bool next = false);
+    // early: the kernel launched before does not change the tree (see kernel_list)
+    void project(int l, int mode, bool early = false);
+    // levels hi..lo in fewer launches; level lo with mode top (mode if top < 0)
+    void project_up(int hi, int lo, int mode, int top = -1, bool early = false);
+    // an iteration begins: leaf copy of levels lmin..L, up-sweep of levels L-1..lo
+    // (level lo with mode top); next: it is not the macro step's first
+    void begin(int lmin, bool next, int lo, int top);
+    void leaf_copy(int lo, int hi, int from, int to); // leaves of levels lo..hi
     void mark_refinements(int la, bool check = false); // check that the tree fits (halt)
     void apply_tree(int la);
     void compact(int lo, int hi);                      // leaf / node / tile lists of levels lo..hi

@@ -11,7 +11,7 @@
 
 namespace mrlt {
 
-enum ProjMode { PM_Q0 = 0, PM_Q1, PM_Q2, PM_REF2, PM_PRJ2, PM_REF3, PM_PRJ3, PM_MID };
+enum ProjMode { PM_Q0 = 0, PM_BEG, PM_Q1, PM_Q2, PM_REF2, PM_PRJ2, PM_REF3, PM_PRJ3, PM_MID };
 
 #define MRLT_GRID_STRIDE(i, n) \
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < (n); i += (long long)gridDim.x * blockDim.x)
@@ -25,6 +25,19 @@ enum ProjMode { PM_Q0 = 0, PM_Q1, PM_Q2, PM_REF2, PM_PRJ2, PM_REF3, PM_PRJ3, PM_
 template <int KIND, class F>
 __device__ __forceinline__ void for_list(const Grid& g, int lo, int hi, F f)
 {
+    const int* list = KIND ? g.inner : g.leaves;
+    if (lo == hi) { // the first entry and the count in one trip (the list has room for every cell)
+        const long long N = g.N[lo], t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+        const int* mine = list + g.off[lo];
+        int e = t0 < N ? mine[t0] : -1;
+        const int total = g.counts[KIND * (LMAX + 1) + lo];
+        for (long long t = t0; t < total; t += (long long)gridDim.x * blockDim.x) {
+            if (t != t0) e = mine[t];
+            if (e < 0 || e >= N) atomicOr(g.err, ERR_INDEX);
+            else f(lo, (long long)e, t);
+        }
+        return;
+    }
     __shared__ int base[LMAX + 2]; // level lo + k starts at base[k]
     __syncthreads();               // base may hold an earlier call's
     if (threadIdx.x < 32) {
@@ -39,7 +52,6 @@ __device__ __forceinline__ void for_list(const Grid& g, int lo, int hi, F f)
         if (k == 0) base[0] = 0;
     }
     __syncthreads();
-    const int* list = KIND ? g.inner : g.leaves;
     const int total = base[hi - lo + 1];
     MRLT_GRID_STRIDE(t, total)
     {
@@ -52,6 +64,34 @@ __device__ __forceinline__ void for_list(const Grid& g, int lo, int hi, F f)
         }
         f(lo + k, id, t);
     }
+}
+
+// for_list for a kernel's whole body, with the tree's share of an entry's work,
+// lookup(l, id), apart from the use(entry) of its result.  early: no kernel
+// that changes the tree directly precedes this launch, so the first entries are
+// looked up before the wait for the predecessor's values (pdl_enter): when this
+// kernel starts, each CTA of its predecessor has itself waited for its own, so
+// whatever built the tree is complete.  Otherwise the wait comes first.
+template <int KIND, class Lookup, class Use>
+__device__ __forceinline__ void kernel_list(const Grid& g, int lo, int hi, bool early, Lookup lookup, Use use)
+{
+    if (!early) {
+        pdl_enter();
+        if (halted(g)) return;
+    }
+    bool waited = !early, stop = false;
+    const auto enter = [&]() {
+        if (waited) return;
+        pdl_enter();
+        waited = true;
+        stop = halted(g);
+    };
+    for_list<KIND>(g, lo, hi, [&](int l, long long id, long long) {
+        auto e = lookup(l, id);
+        enter();
+        if (!stop) use(e);
+    });
+    enter(); // a thread without entries: the kernels after this one rely on its wait
 }
 
 // a node's row of M values: 16-byte accesses where rows are whole vectors
@@ -103,12 +143,15 @@ __device__ __forceinline__ void dev_leaf_copy(const Grid& g, int lo, int hi, int
 // ------------------------------------------------------------ projections
 // Every internal node of level l combines its 2^d children (Eq. 3 mean):
 //  PM_Q0 / PM_Q1 / PM_Q2: plain projection of that field (Alg. 3; GTS stages)
+//  PM_BEG: q^n as an iteration begins, reading the end value of leaf children
+//           (the q^n that the leaf copy gives them in the same launch)
 //  PM_REF2: Alg. 8 -- XH = mean q* (Eq. 17), q* = 2 XH - q^n (Eq. 18)
 //  PM_PRJ2: Alg. 4 -- q* = mean(leaf: Eq. 14 value, internal: Eq. 15 value)
 //  PM_REF3: Alg. 9 -- N1 = mean q**, N3 by Eq. 20, q** by Eq. 21
 //  PM_PRJ3: Alg. 6 -- q** = mean(children at t^n + dt_{l+1}), end value
 //           2 q** - q^n (Eq. 16 with the theta values implied by q**)
-//  PM_MID:  Alg. 3 / Sec. 4.3 refresh of the mid-step level lmin-1
+//  PM_MID:  Alg. 3 / Sec. 4.3 refresh of the mid-step level lmin-1, from its
+//           children's q^n, read likewise
 // one internal node (l, id): the projection of the given mode.  Bound by its
 // dependent trips (list, child slots, rows), so the rows of all children are
 // loaded before any is used; a loop over the variables that stored each before
@@ -116,44 +159,60 @@ __device__ __forceinline__ void dev_leaf_copy(const Grid& g, int lo, int hi, int
 // L = 10 solve on a GB300 (14 k nodes on level 9), this takes 6.0 us.  The
 // roundings are written out: which multiply-adds are fused must not depend on
 // what else the compiler finds to share.
-template <int D, int M, class T>
-__device__ __forceinline__ void project_node(const Grid& g, int l, long long id, int mode)
+// What a projection looks up in the tree: the node's slot, its children's
+// slots, and which of them are leaves.
+template <int D>
+struct NodeRefs {
+    int sl, csl[1 << D];
+    unsigned leaf;
+};
+
+template <int D>
+__device__ __forceinline__ NodeRefs<D> lookup_node(const Grid& g, int l, long long id)
 {
-    constexpr int NCH = 1 << D;
+    NodeRefs<D> r;
     int c[3];
     cell_xyz(g, l, id, c);
-    int csl[NCH];
-    uint8_t cst[NCH];
+    r.leaf = 0;
 #pragma unroll
-    for (int k = 0; k < NCH; ++k) {
+    for (int k = 0; k < (1 << D); ++k) {
         const long long ch = cell_id(g, l + 1, 2 * c[0] + (k & 1), D > 1 ? 2 * c[1] + ((k >> 1) & 1) : 0,
                                      D > 2 ? 2 * c[2] + ((k >> 2) & 1) : 0);
-        cst[k] = status(g, l + 1, ch);
-        csl[k] = slot_of(g, l + 1, ch);
+        r.leaf |= (status(g, l + 1, ch) == 1 ? 1u : 0u) << k;
+        r.csl[k] = slot_of(g, l + 1, ch);
     }
-    const int sl = slot_of(g, l, id);
+    r.sl = slot_of(g, l, id);
+    return r;
+}
+
+template <int D, int M, class T>
+__device__ __forceinline__ void project_node(const Grid& g, const NodeRefs<D>& n, int mode)
+{
+    constexpr int NCH = 1 << D;
+    const int sl = n.sl;
     const int child = mode == PM_Q1 || mode == PM_REF2   ? F_Q1
                       : mode == PM_Q2 || mode == PM_REF3 ? F_Q2
                       : mode == PM_PRJ3                  ? F_QE
-                                                         : F_Q0; // PM_Q0; PM_MID: children at t^n
+                                                         : F_Q0;
+    const int leaf = mode == PM_BEG || mode == PM_MID ? F_QE : child; // a leaf child's q^n is its end value
     T w[NCH][M], acc[M], a0[M], a1[M];
     if (mode == PM_PRJ2) {
         T x[NCH][M];
 #pragma unroll
         for (int k = 0; k < NCH; ++k) {
-            load_row<M, T>(nd<T>(g, F_Q0, csl[k]), w[k]);
-            load_row<M, T>(nd<T>(g, cst[k] != 1 ? F_Q1 : (g.rk == 2 ? F_QE : F_Q2), csl[k]), x[k]);
+            load_row<M, T>(nd<T>(g, F_Q0, n.csl[k]), w[k]);
+            load_row<M, T>(nd<T>(g, !(n.leaf >> k & 1) ? F_Q1 : (g.rk == 2 ? F_QE : F_Q2), n.csl[k]), x[k]);
         }
 #pragma unroll
         for (int k = 0; k < NCH; ++k)
 #pragma unroll
             for (int v = 0; v < M; ++v) {
-                if (cst[k] == 1 && g.rk != 2) w[k][v] = fma(T(4), x[k][v], -mul_rn(T(3), w[k][v]));
+                if ((n.leaf >> k & 1) && g.rk != 2) w[k][v] = fma(T(4), x[k][v], -mul_rn(T(3), w[k][v]));
                 else w[k][v] = T(2) * x[k][v] - w[k][v];
             }
     } else {
 #pragma unroll
-        for (int k = 0; k < NCH; ++k) load_row<M, T>(nd<T>(g, child, csl[k]), w[k]);
+        for (int k = 0; k < NCH; ++k) load_row<M, T>(nd<T>(g, n.leaf >> k & 1 ? leaf : child, n.csl[k]), w[k]);
         if (mode >= PM_REF2) {
             load_row<M, T>(nd<T>(g, F_Q0, sl), a0);
             if (mode == PM_REF3 || mode == PM_MID) load_row<M, T>(nd<T>(g, F_Q1, sl), a1);
@@ -167,7 +226,7 @@ __device__ __forceinline__ void project_node(const Grid& g, int l, long long id,
         acc[v] = acc[v] * T(1.0 / NCH); // the mean
     }
     switch (mode) {
-    case PM_Q0: store_row<M, T>(nd<T>(g, F_Q0, sl), acc); break;
+    case PM_Q0: case PM_BEG: store_row<M, T>(nd<T>(g, F_Q0, sl), acc); break;
     case PM_Q1: case PM_PRJ2: store_row<M, T>(nd<T>(g, F_Q1, sl), acc); break;
     case PM_Q2: store_row<M, T>(nd<T>(g, F_Q2, sl), acc); break;
     case PM_REF2:
@@ -219,52 +278,79 @@ __device__ __forceinline__ void project_node(const Grid& g, int l, long long id,
     }
 }
 
+// An up-sweep of one mode over levels hi..lo in one launch.  Each step of a CTA
+// takes `tops` internal nodes of level lo and projects their internal
+// descendants bottom-up, level by level, with a CTA barrier between levels: a
+// node's projection reads only its own children, which lie in the same subtree.
+// Thread t of a step owns descendant t % sub of top node t / sub on each level
+// (sub = 2^{d (u - lo)} on level u), so 2^{d (hi - lo)} <= blockDim.x, and at
+// most 6 / d levels above lo (kUpDepth).  The nodes of all levels are looked up
+// together (one trip for the list, one for statuses, one for slots), so a level
+// costs the trip of its rows.
+template <int D> constexpr int kUpDepth = 6 / D;
+
+template <int D>
+struct UpRefs {
+    NodeRefs<D> n[kUpDepth<D> + 1];
+    unsigned have; // bit s: this thread projects a node of level lo + s
+};
+
+template <int D>
+__device__ __forceinline__ UpRefs<D> up_lookup(const Grid& g, int hi, int lo, int step)
+{
+    UpRefs<D> r;
+    r.have = 0;
+    const int depth = hi - lo, tops = blockDim.x >> (D * depth), t = threadIdx.x;
+    const int* list = g.inner + g.off[lo];
+    const long long N = g.N[lo];
+    const int cnt = g.counts[LMAX + 1 + lo];
+#pragma unroll
+    for (int s = 0; s <= kUpDepth<D>; ++s) {
+        if (s > depth) continue;
+        const int sub = 1 << (D * s);
+        const long long ti = (long long)step * tops + t / sub;
+        if (t >= tops * sub || ti >= N) continue;
+        const long long top = list[ti]; // with the count: the list has room for every cell
+        if (ti >= cnt) continue;
+        if (top < 0 || top >= N) {
+            atomicOr(g.err, ERR_INDEX);
+            continue;
+        }
+        int tc[3];
+        cell_xyz(g, lo, top, tc);
+        const int q = t % sub, msk = (1 << s) - 1, u = lo + s;
+        const long long id = cell_id(g, u, (tc[0] << s) + (q & msk), D > 1 ? (tc[1] << s) + ((q >> s) & msk) : 0,
+                                     D > 2 ? (tc[2] << s) + (q >> (2 * s)) : 0);
+        if (s && status(g, u, id) != 2) continue;
+        r.have |= 1u << s;
+        r.n[s] = lookup_node<D>(g, u, id);
+    }
+    return r;
+}
+
+// the projections of one step: level lo with mode topmode, the others with mode
+template <int D, int M, class T>
+__device__ __forceinline__ void up_project(const Grid& g, const UpRefs<D>& r, int depth, int mode, int topmode)
+{
+#pragma unroll
+    for (int s = kUpDepth<D>; s >= 0; --s) {
+        if (s > depth) continue;
+        if (r.have >> s & 1) project_node<D, M, T>(g, r.n[s], s ? mode : topmode);
+        if (s) __syncthreads();
+    }
+}
+
+__device__ __forceinline__ int up_steps(const Grid& g, int hi, int lo)
+{
+    const int tops = blockDim.x >> (g.d * (hi - lo));
+    return (g.counts[LMAX + 1 + lo] + tops - 1) / tops;
+}
+
+// one level (the persistent macro-step kernel's phases)
 template <int D, int M, class T>
 __device__ __forceinline__ void dev_project(const Grid& g, int l, int mode)
 {
-    for_list<1>(g, l, l, [&](int, long long id, long long) { project_node<D, M, T>(g, l, id, mode); });
-}
-
-// An up-sweep of one mode over levels hi..lo (hi - lo = depth >= 1) in one
-// launch.  Each step of a CTA takes `tops` internal nodes of level lo and
-// projects their internal descendants bottom-up, level by level, with a CTA
-// barrier between levels: a node's projection reads only its own children,
-// which lie in the same subtree.  Thread t of a step owns descendant t % sub
-// of top node t / sub on each level (sub = 2^{d (m - lo)} on level m), so
-// 2^{d depth} <= blockDim.x is required.  Every node is projected by the same
-// operations as in dev_project.
-template <int D, int M, class T>
-__device__ __forceinline__ void dev_project_up(const Grid& g, int hi, int lo, int mode)
-{
-    const int depth = hi - lo;
-    const int tops = blockDim.x >> (D * depth);
-    const int cnt = g.counts[LMAX + 1 + lo];
-    const int* list = g.inner + g.off[lo];
-    const long long N = g.N[lo];
-    const int nstep = (cnt + tops - 1) / tops;
-    for (int c = blockIdx.x; c < nstep; c += gridDim.x) { // uniform across the CTA
-        for (int u = hi; u >= lo; --u) {
-            const int s = u - lo;
-            const int sub = 1 << (D * s);
-            const int t = threadIdx.x;
-            const int ti = c * tops + t / sub;
-            if (t < tops * sub && ti < cnt) {
-                const long long top = list[ti];
-                if (top < 0 || top >= N) {
-                    atomicOr(g.err, ERR_INDEX);
-                } else {
-                    int tc[3];
-                    cell_xyz(g, lo, top, tc);
-                    const int r = t % sub, msk = (1 << s) - 1;
-                    const long long id = cell_id(g, u, (tc[0] << s) + (r & msk),
-                                                 D > 1 ? (tc[1] << s) + ((r >> s) & msk) : 0,
-                                                 D > 2 ? (tc[2] << s) + (r >> (2 * s)) : 0);
-                    if (status(g, u, id) == 2) project_node<D, M, T>(g, u, id, mode);
-                }
-            }
-            __syncthreads();
-        }
-    }
+    for_list<1>(g, l, l, [&](int, long long id, long long) { project_node<D, M, T>(g, lookup_node<D>(g, l, id), mode); });
 }
 
 // ------------------------------------------------------------ adaptation
@@ -317,70 +403,88 @@ __device__ __forceinline__ void predict_block(const double* b, double* out)
 // Measured on a GB300, per launch: 30 us with weighted sums against 13.8 us in
 // the opening of the 2D Euler L = 10 solve (all depths of remesh), 80 against
 // 11 us at full remeshes of 2D L = 9, 234 against 68 us in the 3D blast at L = 7.
+template <int D>
+struct DetailRefs {
+    static constexpr int NB = D == 1 ? 3 : (D == 2 ? 9 : 27);
+    int l, sl[NB], csl[1 << D];
+    unsigned minus; // block cells that enter negated (an odd count of odd mirrors)
+    long long id;
+};
+
+template <int D>
+__device__ __forceinline__ DetailRefs<D> lookup_detail(const Grid& g, int l, long long id)
+{
+    DetailRefs<D> r;
+    r.l = l;
+    r.id = id;
+    r.minus = 0;
+    int c[3];
+    cell_xyz(g, l, id, c);
+    int q[3][3], neg[3][3]; // in-box coordinate and mirror parity of the neighbours per direction
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) {
+            neg[k][j] = 0;
+            q[k][j] = k < D ? wrap_or_mirror(g, l, k, c[k] + j - 1, neg[k][j]) : 0;
+        }
+    bool missing = false;
+#pragma unroll
+    for (int b = 0; b < DetailRefs<D>::NB; ++b) {
+        const int i = b % 3, j = D > 1 ? b / 3 % 3 : 0, k = D > 2 ? b / 9 : 0;
+        const long long bid = cell_id(g, l, q[0][i], q[1][j], q[2][k]);
+        missing = missing || status(g, l, bid) == 0;
+        r.sl[b] = slot_of(g, l, bid);
+        r.minus |= (unsigned)(neg[0][i] ^ (D > 1 ? neg[1][j] : 0) ^ (D > 2 ? neg[2][k] : 0)) << b;
+    }
+    if (missing && g.eps > 0.0) atomicOr(g.err, ERR_SOURCE);
+#pragma unroll
+    for (int k = 0; k < (1 << D); ++k)
+        r.csl[k] = slot_of(g, l + 1, cell_id(g, l + 1, 2 * c[0] + (k & 1), D > 1 ? 2 * c[1] + ((k >> 1) & 1) : 0,
+                                             D > 2 ? 2 * c[2] + ((k >> 2) & 1) : 0));
+    return r;
+}
+
+template <int D, int M, class T>
+__device__ __forceinline__ void detail_node(const Grid& g, const DetailRefs<D>& e)
+{
+    constexpr int NB = DetailRefs<D>::NB, NCH = 1 << D;
+    uint8_t fl = 0;
+    if (g.eps <= 0.0) {
+        fl = FL_SIG;
+    } else {
+        const double el = eps_level(g, e.l + 1);
+        double nrm = 0.0;
+#pragma unroll(D > 2 ? 1 : M)
+        for (int v = 0; v < M; ++v) {
+            const double sc = __longlong_as_double((long long)g.scale_bits[v]);
+            double b[NB], p[NCH];
+#pragma unroll
+            for (int k = 0; k < NB; ++k) {
+                b[k] = double(nd<T>(g, F_Q0, e.sl[k])[v]);
+                if (e.minus >> k & 1) b[k] = -b[k];
+            }
+            predict_block<D>(b, p);
+            long long mx = 0;
+#pragma unroll
+            for (int k = 0; k < NCH; ++k) {
+                const double d = double(nd<T>(g, F_Q0, e.csl[k])[v]) - p[k];
+                const long long a = __double_as_longlong(d) & 0x7fffffffffffffffLL;
+                if (a > mx && a <= 0x7ff0000000000000LL) mx = a; // a NaN is no detail
+            }
+            nrm = fmax(nrm, __longlong_as_double(mx) / sc);
+        }
+        if (fabs(nrm - el) <= 1e-10 * el || fabs(nrm - 8.0 * el) <= 8e-10 * el) atomicAdd(g.near, 1ull);
+        if (nrm > el) fl |= FL_SIG;
+        if (nrm > 8.0 * el) fl |= FL_BIG;
+    }
+    g.flag[g.off[e.l] + e.id] |= fl;
+}
+
 template <int D, int M, class T>
 __device__ __forceinline__ void dev_detail(const Grid& g, int lo, int hi)
 {
-    constexpr int NB = D == 1 ? 3 : (D == 2 ? 9 : 27), NCH = 1 << D;
-    double sc[M];
-#pragma unroll
-    for (int v = 0; v < M; ++v) sc[v] = __longlong_as_double((long long)g.scale_bits[v]);
-    for_list<1>(g, lo, hi, [&](int l, long long id, long long) {
-        uint8_t fl = 0;
-        if (g.eps <= 0.0) {
-            fl = FL_SIG;
-        } else {
-            const double el = eps_level(g, l + 1);
-            int c[3];
-            cell_xyz(g, l, id, c);
-            int q[3][3], neg[3][3]; // in-box coordinate and mirror parity of the neighbours per direction
-#pragma unroll
-            for (int k = 0; k < 3; ++k)
-#pragma unroll
-                for (int j = 0; j < 3; ++j) {
-                    neg[k][j] = 0;
-                    q[k][j] = k < D ? wrap_or_mirror(g, l, k, c[k] + j - 1, neg[k][j]) : 0;
-                }
-            int sl[NB], csl[NCH];
-            unsigned minus = 0; // block cells that enter negated (an odd count of odd mirrors)
-            bool missing = false;
-#pragma unroll
-            for (int b = 0; b < NB; ++b) {
-                const int i = b % 3, j = D > 1 ? b / 3 % 3 : 0, k = D > 2 ? b / 9 : 0;
-                const long long bid = cell_id(g, l, q[0][i], q[1][j], q[2][k]);
-                missing = missing || status(g, l, bid) == 0;
-                sl[b] = slot_of(g, l, bid);
-                minus |= (unsigned)(neg[0][i] ^ (D > 1 ? neg[1][j] : 0) ^ (D > 2 ? neg[2][k] : 0)) << b;
-            }
-            if (missing) atomicOr(g.err, ERR_SOURCE);
-#pragma unroll
-            for (int k = 0; k < NCH; ++k)
-                csl[k] = slot_of(g, l + 1, cell_id(g, l + 1, 2 * c[0] + (k & 1), D > 1 ? 2 * c[1] + ((k >> 1) & 1) : 0,
-                                                   D > 2 ? 2 * c[2] + ((k >> 2) & 1) : 0));
-            double nrm = 0.0;
-#pragma unroll(D > 2 ? 1 : M)
-            for (int v = 0; v < M; ++v) {
-                double b[NB], p[NCH];
-#pragma unroll
-                for (int k = 0; k < NB; ++k) {
-                    b[k] = double(nd<T>(g, F_Q0, sl[k])[v]);
-                    if (minus >> k & 1) b[k] = -b[k];
-                }
-                predict_block<D>(b, p);
-                long long mx = 0;
-#pragma unroll
-                for (int k = 0; k < NCH; ++k) {
-                    const double d = double(nd<T>(g, F_Q0, csl[k])[v]) - p[k];
-                    const long long a = __double_as_longlong(d) & 0x7fffffffffffffffLL;
-                    if (a > mx && a <= 0x7ff0000000000000LL) mx = a; // a NaN is no detail
-                }
-                nrm = fmax(nrm, __longlong_as_double(mx) / sc[v]);
-            }
-            if (fabs(nrm - el) <= 1e-10 * el || fabs(nrm - 8.0 * el) <= 8e-10 * el) atomicAdd(g.near, 1ull);
-            if (nrm > el) fl |= FL_SIG;
-            if (nrm > 8.0 * el) fl |= FL_BIG;
-        }
-        g.flag[g.off[l] + id] |= fl;
-    });
+    for_list<1>(g, lo, hi, [&](int l, long long id, long long) { detail_node<D, M, T>(g, lookup_detail<D>(g, l, id)); });
 }
 
 template <int D>
@@ -1088,67 +1192,86 @@ __device__ __forceinline__ void level_tile_list(const Grid& g, int l)
 // children at once.  One face, variable and child after the other took 40 us
 // per launch over the opening of the 2D Euler L = 10 solve on a GB300 (73 k
 // leaves), and 142 us in the 3D blast at L = 7; this takes 13 and 36 us.
+template <int D>
+struct RefluxRefs {
+    unsigned finer; // faces to an internal node
+    int l, c[3], sl;
+};
+
+template <int D>
+__device__ __forceinline__ RefluxRefs<D> lookup_reflux(const Grid& g, int l, long long id)
+{
+    RefluxRefs<D> r;
+    r.l = l;
+    cell_xyz(g, l, id, r.c);
+    uint8_t st[2 * D];
+#pragma unroll
+    for (int fi = 0; fi < 2 * D; ++fi) {
+        int nb[3] = {r.c[0], r.c[1], r.c[2]};
+        st[fi] = in_box(g, l, fi >> 1, r.c[fi >> 1] + (fi & 1 ? 1 : -1), &nb[fi >> 1])
+                     ? status(g, l, cell_id(g, l, nb[0], nb[1], nb[2]))
+                     : 0;
+    }
+    r.sl = slot_of(g, l, id);
+    r.finer = 0;
+#pragma unroll
+    for (int fi = 0; fi < 2 * D; ++fi) r.finer |= (st[fi] == 2 ? 1u : 0u) << fi;
+    return r;
+}
+
+template <int D, int M, class T>
+__device__ __forceinline__ void reflux_leaf(const Grid& g, const RefluxRefs<D>& e)
+{
+    constexpr int NT = 1 << (D - 1);
+    if (!e.finer) return;
+    const int l = e.l;
+    const int* c = e.c;
+    double* rc = regs(g.rg, g, e.sl);
+    T q[M];
+    load_row<M, T>(nd<T>(g, F_QE, e.sl), q);
+    for (unsigned finer = e.finer; finer; finer &= finer - 1) {
+        const int fi = __ffs(finer) - 1, k = fi >> 1, side = (fi & 1) ? 1 : -1;
+        const int opp = 2 * k + (side > 0 ? 0 : 1);
+        int nk; // the neighbour's coordinate along k
+        in_box(g, l, k, (k == 0 ? c[0] : (k == 1 ? c[1] : c[2])) + side, &nk);
+        double* rf[NT];
+#pragma unroll
+        for (int tt = 0; tt < NT; ++tt) {
+            int p[3] = {0, 0, 0}, bit = 0;
+#pragma unroll
+            for (int j = 0; j < D; ++j) {
+                if (j == k) p[j] = 2 * nk + (side > 0 ? 0 : 1);
+                else p[j] = 2 * c[j] + ((tt >> bit++) & 1);
+            }
+            const long long ch = cell_id(g, l + 1, p[0], p[1], p[2]);
+            if (status(g, l + 1, ch) != 1) atomicOr(g.err, ERR_REFLUX);
+            rf[tt] = regs(g.rg, g, slot_of(g, l + 1, ch)) + opp * M;
+        }
+        double r[NT][M], own[M];
+        const double none[M] = {};
+        load_row<M, double>(rc + fi * M, own);
+#pragma unroll
+        for (int tt = 0; tt < NT; ++tt) load_row<M, double>(rf[tt], r[tt]);
+        const double idx = g.rdx[l][k];
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+            double sum = 0.0;
+#pragma unroll
+            for (int tt = 0; tt < NT; ++tt) sum += r[tt][v];
+            // the correction from the FP64 registers, rounded to T once
+            q[v] = T(double(q[v]) + side * (own[v] - sum * (1.0 / NT)) * idx);
+        }
+        store_row<M, double>(rc + fi * M, none);
+#pragma unroll
+        for (int tt = 0; tt < NT; ++tt) store_row<M, double>(rf[tt], none);
+    }
+    store_row<M, T>(nd<T>(g, F_QE, e.sl), q);
+}
+
 template <int D, int M, class T>
 __device__ __forceinline__ void dev_reflux(const Grid& g, int lo, int hi)
 {
-    constexpr int NT = 1 << (D - 1);
-    for_list<0>(g, lo, hi, [&](int l, long long id, long long) {
-        int c[3];
-        cell_xyz(g, l, id, c);
-        uint8_t st[2 * D];
-#pragma unroll
-        for (int fi = 0; fi < 2 * D; ++fi) {
-            int nb[3] = {c[0], c[1], c[2]};
-            st[fi] = in_box(g, l, fi >> 1, c[fi >> 1] + (fi & 1 ? 1 : -1), &nb[fi >> 1])
-                         ? status(g, l, cell_id(g, l, nb[0], nb[1], nb[2]))
-                         : 0;
-        }
-        unsigned finer = 0; // faces to an internal node
-#pragma unroll
-        for (int fi = 0; fi < 2 * D; ++fi) finer |= (st[fi] == 2 ? 1u : 0u) << fi;
-        if (!finer) return;
-        const int sl = slot_of(g, l, id);
-        double* rc = regs(g.rg, g, sl);
-        T q[M];
-        load_row<M, T>(nd<T>(g, F_QE, sl), q);
-        for (; finer; finer &= finer - 1) {
-            const int fi = __ffs(finer) - 1, k = fi >> 1, side = (fi & 1) ? 1 : -1;
-            const int opp = 2 * k + (side > 0 ? 0 : 1);
-            int nk; // the neighbour's coordinate along k
-            in_box(g, l, k, (k == 0 ? c[0] : (k == 1 ? c[1] : c[2])) + side, &nk);
-            double* rf[NT];
-#pragma unroll
-            for (int tt = 0; tt < NT; ++tt) {
-                int p[3] = {0, 0, 0}, bit = 0;
-#pragma unroll
-                for (int j = 0; j < D; ++j) {
-                    if (j == k) p[j] = 2 * nk + (side > 0 ? 0 : 1);
-                    else p[j] = 2 * c[j] + ((tt >> bit++) & 1);
-                }
-                const long long ch = cell_id(g, l + 1, p[0], p[1], p[2]);
-                if (status(g, l + 1, ch) != 1) atomicOr(g.err, ERR_REFLUX);
-                rf[tt] = regs(g.rg, g, slot_of(g, l + 1, ch)) + opp * M;
-            }
-            double r[NT][M], own[M];
-            const double none[M] = {};
-            load_row<M, double>(rc + fi * M, own);
-#pragma unroll
-            for (int tt = 0; tt < NT; ++tt) load_row<M, double>(rf[tt], r[tt]);
-            const double idx = g.rdx[l][k];
-#pragma unroll
-            for (int v = 0; v < M; ++v) {
-                double sum = 0.0;
-#pragma unroll
-                for (int tt = 0; tt < NT; ++tt) sum += r[tt][v];
-                // the correction from the FP64 registers, rounded to T once
-                q[v] = T(double(q[v]) + side * (own[v] - sum * (1.0 / NT)) * idx);
-            }
-            store_row<M, double>(rc + fi * M, none);
-#pragma unroll
-            for (int tt = 0; tt < NT; ++tt) store_row<M, double>(rf[tt], none);
-        }
-        store_row<M, T>(nd<T>(g, F_QE, sl), q);
-    });
+    for_list<0>(g, lo, hi, [&](int l, long long id, long long) { reflux_leaf<D, M, T>(g, lookup_reflux<D>(g, l, id)); });
 }
 
 // ------------------------------------------------------------ reductions
