@@ -11,6 +11,7 @@
 #include <new>
 #include <string>
 #include <vector>
+#include <atomic>
 #include <chrono>
 #include <mutex>
 #include <thread>
@@ -47,6 +48,7 @@ struct mr_solver {
     bool unchecked = false;         // iterations launched since the last check point
     long long halts = 0;            // halts recovered (statistics)
     long long reserved = 0;         // mr_reserve_nodes: capacity floor
+    bool copy_input = false;        // initial data are in short-lived memory (see load_finest)
     double t = 0.0, dt = 0.0;
     long long iters = 0, macros = 0, pos = 0, stage_launches = 0;
     bool reg = false;
@@ -1000,7 +1002,53 @@ mr_status cfl_dt(mr_solver* h, double* dt)
     return MR_OK;
 }
 
-mr_status init_state(mr_solver* h, const double* q0)
+// Can kernels read any host memory through the host's own page tables (a GPU
+// coherent with its host over NVLink-C2C, as on GB300)?  Looked up once per
+// device.
+bool reads_host_memory()
+{
+    static std::atomic<int> known[kMaxPoolDevices] = {}; // 0 not looked up, 1 no, 2 yes
+    int dev = 0, any = 0, tables = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxPoolDevices) return false;
+    if (!known[dev].load()) {
+        const bool ok = cudaDeviceGetAttribute(&any, cudaDevAttrPageableMemoryAccess, dev) == cudaSuccess &&
+                        cudaDeviceGetAttribute(&tables, cudaDevAttrPageableMemoryAccessUsesHostPageTables, dev) ==
+                            cudaSuccess &&
+                        any && tables;
+        cudaGetLastError();
+        known[dev].store(ok ? 2 : 1);
+    }
+    return known[dev].load() == 2;
+}
+
+// The caller's finest data into q^n of the finest nodes.  Large data are read in
+// place where kernels can: a copy from pageable memory goes through the driver's
+// staging buffers at the speed of one host thread, so that with data not in the
+// host's caches a 3D solve at L = 8 (671 MB of data, mixed, 32 iterations) took
+// 139 ms on a GB300 with the copy and 50 ms without; at 8 MB (2D, L = 9) both
+// ways take the same.  Not for memory that is released right after
+// (h->copy_input): unmapping what the GPU has read costs more than the copy (a
+// server mix of 12 requests 65 against 60 ms).  The caller's memory is read
+// until the stream has been waited for, before the call returns.
+constexpr size_t kReadInPlace = 16u << 20;
+
+mr_status load_finest(mr_solver* h, const double* q0)
+{
+    Grid& g = h->K.g;
+    const size_t bytes = (size_t)g.N[g.L] * g.m * sizeof(double);
+    if (bytes >= kReadInPlace && !h->copy_input && reads_host_memory()) {
+        h->K.store_finest(q0);
+        return MR_OK;
+    }
+    double* d_q = nullptr; // through a transient device buffer
+    MR_TRY(scratch(h, &d_q, (size_t)g.N[g.L] * g.m));
+    MR_CK(cudaMemcpyAsync(d_q, q0, bytes, cudaMemcpyHostToDevice, h->stream));
+    h->K.store_finest(d_q);
+    MR_CK(cudaFreeAsync(d_q, h->stream));
+    return MR_OK;
+}
+
+mr_status fresh_state(mr_solver* h, const double* q0)
 {
     Grid& g = h->K.g;
     const int m = g.m;
@@ -1021,11 +1069,7 @@ mr_status init_state(mr_solver* h, const double* q0)
     for (int l = g.lb; l <= g.L; ++l)
         MR_CK(cudaMemsetAsync(g.st + g.off[l], l < g.L ? 2 : 1, (size_t)g.N[l], h->stream));
     h->K.slots_full(h->ntot);
-    double* d_q = nullptr; // finest data through a transient double buffer, stored in the fields' type
-    MR_TRY(scratch(h, &d_q, (size_t)g.N[g.L] * m));
-    MR_CK(cudaMemcpyAsync(d_q, q0, (size_t)g.N[g.L] * m * sizeof(double), cudaMemcpyHostToDevice, h->stream));
-    h->K.store_finest(d_q);
-    MR_CK(cudaFreeAsync(d_q, h->stream));
+    MR_TRY(load_finest(h, q0));
     h->K.compact(g.lb, g.L);
     for (int l = g.L - 1; l >= g.lb; --l) h->K.project(l, PM_Q0);
     if (h->cfg.adapt_mode != MR_ADAPT_NEVER) MR_TRY(adapt(h, g.lb));
@@ -1037,11 +1081,14 @@ mr_status init_state(mr_solver* h, const double* q0)
     return fit_new_tree(h);
 }
 
+mr_status init_state(mr_solver* h, const double* q0)
+{
+    const mr_status r = fresh_state(h, q0);
+    if (r != MR_OK) cudaStreamSynchronize(h->stream); // a kernel may still be reading q0
+    return r;
+}
+
 } // namespace
-
-extern "C" {
-
-} // extern "C"
 
 namespace {
 
@@ -1147,7 +1194,11 @@ mr_status layout_alloc(mr_solver* h, const mr_config* cfg)
 
 extern "C" {
 
-mr_status mr_create(const mr_config* cfg, const double* q0, void* cuda_stream, mr_solver** out)
+} // extern "C"
+
+namespace {
+
+mr_status create(const mr_config* cfg, const double* q0, bool copy_input, void* cuda_stream, mr_solver** out)
 {
     if (!out) return MR_E_INVALID;
     *out = nullptr;
@@ -1167,6 +1218,7 @@ mr_status mr_create(const mr_config* cfg, const double* q0, void* cuda_stream, m
     mr_solver* h = new (std::nothrow) mr_solver();
     if (!h) return MR_E_NOMEM;
     h->cfg = *cfg;
+    h->copy_input = copy_input;
     h->stream = (cudaStream_t)cuda_stream;
     h->K.st = h->stream;
     mr_status r = layout_alloc(h, cfg);
@@ -1178,6 +1230,15 @@ mr_status mr_create(const mr_config* cfg, const double* q0, void* cuda_stream, m
     }
     *out = h;
     return MR_OK;
+}
+
+} // namespace
+
+extern "C" {
+
+mr_status mr_create(const mr_config* cfg, const double* q0, void* cuda_stream, mr_solver** out)
+{
+    return create(cfg, q0, false, cuda_stream, out);
 }
 
 mr_status mr_reset(mr_solver* h, const double* q0)
@@ -1313,7 +1374,8 @@ mr_status mr_create_from_state(const mr_config* cfg, long long n_leaves, const i
     c0.adapt_mode = MR_ADAPT_NEVER;
     std::vector<double> zeros((size_t)m * NL, 0.0);
     mr_solver* h = nullptr;
-    MR_TRY(mr_create(&c0, zeros.data(), cuda_stream, &h));
+    MR_TRY(create(&c0, zeros.data(), true, cuda_stream, &h));
+    h->copy_input = false; // a later mr_reset brings the caller's own data
     h->cfg = *cfg;
     mr_status r = mr_set_tree(h, map.data());
     Grid& g = h->K.g;
@@ -2001,7 +2063,7 @@ mr_status admit(mr_server* s)
             cudaEventCreateWithFlags(&q->ev, cudaEventDisableTiming) != cudaSuccess ||
             cudaEventCreateWithFlags(&q->fin, cudaEventDisableTiming) != cudaSuccess)
             r = MR_E_CUDA;
-        if (r == MR_OK) r = mr_create(&q->cfg, q->q0.data(), q->st, &q->h);
+        if (r == MR_OK) r = create(&q->cfg, q->q0.data(), true, q->st, &q->h);
         q->q0.clear();
         q->q0.shrink_to_fit();
         ++k;

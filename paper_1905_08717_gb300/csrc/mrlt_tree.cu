@@ -455,26 +455,29 @@ void Launcher::set_leaves(const int* keys, const double* vals, long long count)
     ++n;
 }
 
-// finest-level data (host layout [v][cell], uploaded as double) stored in
-// q^n of the finest nodes, in the fields' type
-template <class T>
-__global__ void k_store_finest(Grid g, const double* src)
+// finest-level data (double, host layout [v][cell], in device memory or read
+// from the host's) stored in q^n of the finest nodes, in the fields' type
+template <int M, class T>
+__global__ void k_store_finest(const __grid_constant__ Grid g, const double* src)
 {
     pdl_enter();
     const long long N = g.N[g.L];
     GRID_STRIDE(id, N)
     {
-        T* q0 = nd<T>(g, F_Q0, slot_of(g, g.L, id));
-        for (int v = 0; v < g.m; ++v) q0[v] = T(src[v * N + id]);
+        T q[M];
+#pragma unroll
+        for (int v = 0; v < M; ++v) q[v] = T(src[v * N + id]);
+        store_row<M, T>(nd<T>(g, F_Q0, slot_of(g, g.L, id)), q);
     }
 }
 
-void Launcher::store_finest(const double* src)
+template <int D, int M>
+static void store_finest_dm(Launcher& L, const double* src)
 {
-    if (g.prec) pdl_launch(k_store_finest<float>, blocks_dense(g.N[g.L]), NTHREADS, 0, st, g, src);
-    else pdl_launch(k_store_finest<double>, blocks_dense(g.N[g.L]), NTHREADS, 0, st, g, src);
-    ++n;
+    MRLT_T_LAUNCH(L, blocks_dense(L.g.N[L.g.L]), (L.g, src), k_store_finest<M);
+    ++L.n;
 }
+void Launcher::store_finest(const double* src) { MRLT_DM_DISPATCH(store_finest_dm, *this, src); }
 
 // every cell of levels lb..L a node, in level and cell order from slot 1 on:
 // the full tree of a new solver; the free stack holds the rest
