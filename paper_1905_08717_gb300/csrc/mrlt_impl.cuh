@@ -410,10 +410,13 @@ __device__ __forceinline__ long long ordered_bits(double a) // ordered as the va
 __device__ __forceinline__ bool less(double a, double b) { return ordered_bits(a) < ordered_bits(b); }
 __device__ __forceinline__ bool negative(double a) { return __double2hiint(a) < 0; } // sign bit
 __device__ __forceinline__ bool positive(double a) { return __double_as_longlong(a) > 0; } // and not +0
-__device__ __forceinline__ bool below_abs(double a, double b) // |a| < |b|
+// bits of |a|, one place up: ordered as the magnitudes are.  (Masking the sign bit
+// instead is recognised as fabs, which is an FP64 instruction.)
+__device__ __forceinline__ unsigned long long abs_bits(double a)
 {
-    return (__double_as_longlong(a) & 0x7fffffffffffffffLL) < (__double_as_longlong(b) & 0x7fffffffffffffffLL);
+    return (unsigned long long)__double_as_longlong(a) << 1;
 }
+__device__ __forceinline__ bool below_abs(double a, double b) { return abs_bits(a) < abs_bits(b); } // |a| < |b|
 
 // A product and a sum rounded by themselves, never contracted into a
 // multiply-add.  Where an expression could be contracted in two ways, the one
@@ -599,11 +602,13 @@ __device__ __forceinline__ void ausm_plus64(const Grid& g, int k, const double* 
 // run one way) the flux is sum over the sides of w (F(U) - s U), s the
 // other... outer speed of that side, i.e. U (w (u_n - s)) plus w times the pressure terms.
 // The two mass fluxes rho w (u_n - s) carry momentum and kinetic energy, so
-// neither the conservative states nor the physical fluxes are formed: about 80
-// FP64 operations per face with the reconstruction instead of 135.  Measured on
-// a GB300 together with child() and the comparisons above, mean stage-2 launch:
+// neither the conservative states nor the physical fluxes are formed.  Counted
+// by the hardware on a full grid (2D, all leaves): 214 FP64 operations per leaf
+// and stage, at 77% of the FP64 units' time.  Measured on a GB300 when this, the
+// comparisons above and child() replaced the general forms, mean stage-2 launch:
 // 2D Euler L = 10 from 43.9 to 35.8 us on level 10 and 33.3 to 24.9 us on level
-// 9, 3D blast L = 7 from 308 to 243 us on level 7.
+// 9, 3D blast L = 7 from 308 to 243 us on level 7; recip, recip_sqrt and abs_bits
+// then took the full-grid launch (262 k leaves) from 155 to 133 us.
 template <int D, int M>
 __device__ __forceinline__ void hll64(const Grid& g, int k, const double* PL, const double* PR, double* F)
 {

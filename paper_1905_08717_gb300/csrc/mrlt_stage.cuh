@@ -857,24 +857,17 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
                     F);
             }
         }
-        // mean of the sub-face fluxes of a face (every lane takes part in the
-        // shuffles; plain-face lanes keep their own flux)
-        if constexpr (NTS == 2) {
+        // mean of the sub-face fluxes of a face: in the warps that hold any (their
+        // every lane takes part in the shuffles; plain faces keep their own flux)
+        if (NTS > 1 && base + 32 * warp < nsub) {
 #pragma unroll
             for (int v = 0; v < M; ++v) {
-                const R other = __shfl_xor_sync(0xffffffffu, F[v], 1);
-                if (isSub && t == 0) sF[v][f] = (F[v] + other) * R(0.5);
-                else if (act && !isSub) sF[v][f] = F[v];
+                R sum = F[v] + __shfl_xor_sync(0xffffffffu, F[v], 1);
+                if (NTS == 4) sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+                if (isSub) F[v] = sum * R(1.0 / NTS);
             }
-        } else if constexpr (NTS == 4) {
-#pragma unroll
-            for (int v = 0; v < M; ++v) {
-                const R pair = F[v] + __shfl_xor_sync(0xffffffffu, F[v], 1);
-                const R quad = pair + __shfl_xor_sync(0xffffffffu, pair, 2);
-                if (isSub && t == 0) sF[v][f] = quad * R(0.25);
-                else if (act && !isSub) sF[v][f] = F[v];
-            }
-        } else if (act) {
+        }
+        if (act && t == 0) {
 #pragma unroll
             for (int v = 0; v < M; ++v) sF[v][f] = F[v];
         }

@@ -465,14 +465,14 @@ __device__ __forceinline__ void detail_node(const Grid& g, const DetailRefs<D>& 
                 if (e.minus >> k & 1) b[k] = -b[k];
             }
             predict_block<D>(b, p);
-            long long mx = 0;
+            unsigned long long mx = 0;
 #pragma unroll
             for (int k = 0; k < NCH; ++k) {
                 const double d = double(nd<T>(g, F_Q0, e.csl[k])[v]) - p[k];
-                const long long a = __double_as_longlong(d) & 0x7fffffffffffffffLL;
-                if (a > mx && a <= 0x7ff0000000000000LL) mx = a; // a NaN is no detail
+                const unsigned long long a = abs_bits(d);
+                if (a > mx && a <= 0x7ff0000000000000ull << 1) mx = a; // a NaN is no detail
             }
-            nrm = fmax(nrm, __longlong_as_double(mx) / sc);
+            nrm = fmax(nrm, __longlong_as_double((long long)(mx >> 1)) / sc);
         }
         if (fabs(nrm - el) <= 1e-10 * el || fabs(nrm - 8.0 * el) <= 8e-10 * el) atomicAdd(g.near, 1ull);
         if (nrm > el) fl |= FL_SIG;
