@@ -95,24 +95,25 @@ __global__ void k_detail(const __grid_constant__ Grid g, int lo, int hi)
 
 // Desired and admissible refinements in one pass: desire reads only the detail
 // bits, which the stores of the refinement bit keep.
-// check: this launch finalises the refinement flags (a remesh at level
-// la = L-1 has no closure), so it also checks that the new tree fits.
+// count: the tree's size is checked (room_count); last: this launch finalises
+// the flags (a remesh at level la = L-1 has no closure) and decides.
 template <int D>
-__global__ void k_mark(const __grid_constant__ Grid g, int lo, int hi, int la, bool check)
+__global__ void k_mark(const __grid_constant__ Grid g, int lo, int hi, int la, bool count, bool last)
 {
     MRLT_ENTER(g);
-    dev_mark<D>(g, lo, hi, la);
-    if (check) room_decide(g, refined_here(g, la), la);
+    const int c = dev_mark<D>(g, lo, hi, la);
+    if (last) room_decide(g, c, la);
+    else if (count) room_count(g, c);
 }
 
-// check: the last closure (level l-1 = la), which also checks that the new
-// tree fits; its threads read back the level-la flags they wrote themselves
+// last: the last closure (level l-1 = la)
 template <int D>
-__global__ void k_close(const __grid_constant__ Grid g, int l, bool check)
+__global__ void k_close(const __grid_constant__ Grid g, int l, bool count, bool last)
 {
     MRLT_ENTER(g);
-    dev_close<D>(g, l);
-    if (check) room_decide(g, refined_here(g, l - 1), l - 1);
+    const int c = dev_close<D>(g, l);
+    if (last) room_decide(g, c, l - 1);
+    else if (count) room_count(g, c);
 }
 
 template <int D, int M, class T>
@@ -363,10 +364,10 @@ static void adapt_dm(Launcher& L, int la, bool check)
     const int hi = g.L - 1; // levels whose nodes may own children
     if (g.prec) pdl_launch(k_detail<D, M, float>, blocks_list(g, hi), NTHREADS, 0, L.st, g, la, hi);
     else pdl_launch(k_detail<D, M, double>, blocks_list(g, hi), NTHREADS, 0, L.st, g, la, hi);
-    pdl_launch(k_mark<D>, blocks_step(g, hi), NTHREADS, 0, L.st, g, la, hi, la, check && la == hi);
+    pdl_launch(k_mark<D>, blocks_step(g, hi), NTHREADS, 0, L.st, g, la, hi, la, check, check && la == hi);
     L.n += 2;
     for (int l = g.L - 1; l > la; --l, ++L.n)
-        pdl_launch(k_close<D>, blocks_step(g, l - 1), NTHREADS, 0, L.st, g, l, check && l == la + 1);
+        pdl_launch(k_close<D>, blocks_step(g, l - 1), NTHREADS, 0, L.st, g, l, check, check && l == la + 1);
 }
 
 
@@ -503,23 +504,19 @@ void Launcher::slots_full(long long ntot)
     ++n;
 }
 
-// Refinement flags over cells [from, to), added into *out: after the
-// closure of an adaptation at level la every flagged cell of levels
-// la..L-1 owns 2^d nodes of the new tree.
-__global__ void k_count_ref(const __grid_constant__ Grid g, long long from, long long to, int* out)
+// Refinement flags of levels la..L-1, added into *out: after the closure of an
+// adaptation at level la every flagged cell owns 2^d nodes of the new tree.
+__global__ void k_count_ref(const __grid_constant__ Grid g, int la, int* out)
 {
     MRLT_ENTER(g);
-    int c = 0;
-    GRID_STRIDE(i, to - from) c += (g.flag[from + i] & FL_REF) ? 1 : 0;
-    c = __reduce_add_sync(0xffffffffu, c);
+    const int c = __reduce_add_sync(0xffffffffu, refined_here(g, la));
     if ((threadIdx.x & 31) == 0 && c) atomicAdd(out, c);
 }
 
 void Launcher::count_refined(int la, int* out)
 {
     cudaMemsetAsync(out, 0, sizeof(int), st);
-    const long long from = g.off[la], to = g.off[g.L];
-    pdl_launch(k_count_ref, blocks_dense(to - from), NTHREADS, 0, st, g, from, to, out);
+    pdl_launch(k_count_ref, blocks_dense((g.off[g.L] - g.off[la]) / kStep), NTHREADS, 0, st, g, la, out);
     ++n;
 }
 

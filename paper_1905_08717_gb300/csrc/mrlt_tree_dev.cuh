@@ -711,10 +711,12 @@ __device__ __forceinline__ void refine16(uint8_t* f, unsigned m)
 }
 
 // Refinements of levels lo..hi: desired and admissible.  A step's stores keep
-// the detail bits that other threads read.
+// the detail bits that other threads read.  Returns how many cells this thread
+// flagged.
 template <int D>
-__device__ __forceinline__ void dev_mark(const Grid& g, int lo, int hi, int la)
+__device__ __forceinline__ int dev_mark(const Grid& g, int lo, int hi, int la)
 {
+    int count = 0;
     for (int l = lo; l <= hi; ++l) {
         uint8_t* fl = g.flag + g.off[l];
         int c[3];
@@ -722,7 +724,10 @@ __device__ __forceinline__ void dev_mark(const Grid& g, int lo, int hi, int la)
             MRLT_GRID_STRIDE(id, g.N[l])
             {
                 cell_xyz(g, l, id, c);
-                if (desired<D>(g, l, c, la) && allowed<D>(g, l, c, la)) fl[id] |= FL_REF;
+                if (desired<D>(g, l, c, la) && allowed<D>(g, l, c, la)) {
+                    fl[id] |= FL_REF;
+                    ++count;
+                }
             }
         } else {
             MRLT_GRID_STRIDE(s, g.N[l] / kStep)
@@ -731,16 +736,20 @@ __device__ __forceinline__ void dev_mark(const Grid& g, int lo, int hi, int la)
                 unsigned m = desired16<D>(g, l, c, la);
                 if (m) m = allowed16<D>(g, l, c, la, m);
                 if (m) refine16(fl + s * kStep, m);
+                count += __popc(m);
             }
         }
     }
+    return count;
 }
 
 // grading closure, one level: refining (l, i) refines (l-1, floor(i/2) + delta)
-// for |delta|_inf <= 1 -- gathered at the coarse node
+// for |delta|_inf <= 1 -- gathered at the coarse node.  Returns how many cells
+// this thread flagged.
 template <int D>
-__device__ __forceinline__ void dev_close(const Grid& g, int l)
+__device__ __forceinline__ int dev_close(const Grid& g, int l)
 {
+    int count = 0;
     const int pl = l - 1;
     uint8_t* fp = g.flag + g.off[pl];
     const uint8_t* fc = g.flag + g.off[l];
@@ -763,9 +772,12 @@ __device__ __forceinline__ void dev_close(const Grid& g, int l)
                     if (fc[cid] & FL_REF) hit = true;
                 }
             }
-            if (hit) fp[pid] |= FL_REF;
+            if (hit) {
+                fp[pid] |= FL_REF;
+                ++count;
+            }
         }
-        return;
+        return count;
     }
     MRLT_GRID_STRIDE(s, g.N[pl] / kStep)
     {
@@ -795,20 +807,27 @@ __device__ __forceinline__ void dev_close(const Grid& g, int l)
             }
         const unsigned hit = (m | m >> 1 | m >> 2) & 0xffffu & ~own;
         if (hit) refine16(fp + s * kStep, hit);
+        count += __popc(hit);
     }
+    return count;
 }
 
-// Does the tree flagged by a remesh at level la fit the
-// node arrays?  Each thread of the kernel that finalises the flags counted
-// `c` refined cells (the kernel's cells of levels la..L-1 in one flat
-// grid-stride range over them); the blocks add their counts into room[0].
+// Does the tree flagged by a remesh at level la fit the node arrays?  The
+// threads of its mark and closure passes count the cells c that they flag, and
+// the blocks add their counts into room[0] (counting the flags again in the last
+// pass, which has few blocks when la is a coarse level, took up to 20 us).
 // The new tree has 2^d nodes above level la per refined cell, and the slots
 // it may take are the free ones plus those of the nodes above level la now
-// (the remesh releases them first).  The last block to finish (ticket
-// room[3]) decides: short of slots, the solver halts at this iteration (room[4],
-// counted on by its first kernel), room[1] = it + 1, room[2] = the nodes of
-// the new tree (see halted()).
-// Called by every thread of the block.
+// (the remesh releases them first).  The last block of the last pass to finish
+// (ticket room[3]) decides: short of slots, the solver halts at this iteration
+// (room[4], counted on by its first kernel), room[1] = it + 1, room[2] = the
+// nodes of the new tree (see halted()).  Called by every thread of the block.
+__device__ __forceinline__ void room_count(const Grid& g, int c)
+{
+    c = __reduce_add_sync(0xffffffffu, c);
+    if ((threadIdx.x & 31) == 0 && c) atomicAdd(&g.room[0], c);
+}
+
 __device__ __forceinline__ void room_decide(const Grid& g, int c, int la)
 {
     __shared__ int blk;
@@ -836,8 +855,7 @@ __device__ __forceinline__ void room_decide(const Grid& g, int c, int la)
     }
 }
 
-// refined cells among this thread's cells of levels la..L-1, in the grid-stride
-// order of the passes that flag level la (its other levels are complete)
+// refined cells among this thread's share of levels la..L-1
 __device__ __forceinline__ int refined_here(const Grid& g, int la)
 {
     int c = 0;
