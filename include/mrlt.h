@@ -183,7 +183,7 @@ mr_status mr_set_grid_cap(mr_solver* h, int ctas);
 /* How fine iterations are launched.  MR_LAUNCH_GRAPH (the default) launches
  * one kernel per phase of an iteration (projections, refreshes and stage
  * sweeps per level, the adaptation passes, compaction, reflux; Algs. 3-9),
- * whole macro steps replayed as a CUDA graph; batch instances and served
+ * whole macro steps replayed from captured CUDA graphs; batch instances and served
  * requests always use it, because they run concurrently on their own streams.
  * MR_LAUNCH_PERSISTENT runs the iterations of a macro step in one cooperative
  * launch of a persistent kernel whose CTAs all stay resident, the phases
@@ -299,8 +299,8 @@ mr_status mr_release_cached_memory(void);
  * initial data) advanced together.  The paper treats one problem at a time;
  * batching is this library's way of filling a GPU with problems that are
  * each too small for it.  Every instance is an ordinary solver with its own
- * device memory and its own internal CUDA stream; one macro step of an
- * instance is a CUDA graph (captured once per instance), so the instances'
+ * device memory and its own internal CUDA stream; macro steps of an
+ * instance replay CUDA graphs (captured once per instance), so the instances'
  * kernels overlap on the GPU while the host only picks each instance's CFL
  * step (Sec. 4, Eq. 13) and launches its graph. */
 typedef struct mr_batch mr_batch;

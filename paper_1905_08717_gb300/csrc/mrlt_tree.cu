@@ -134,10 +134,12 @@ __global__ void k_release_apply(const __grid_constant__ Grid g, int la)
     dev_apply<D, M, T, NTHREADS>(g, la, la);
 }
 
-// A small tree (at most kOneBlock cells on the finest level: one step per thread)
-// is flagged and installed by one block each, its levels separated by barriers
-// instead of launches.  Measured on a GB300: a 1D Burgers solve at L = 10, 512
-// iterations, 17.8 ms with a launch per level and 17.1 ms so.
+// A small 1D tree (at most kOneBlock cells on the finest level: one step per
+// thread) is flagged and installed by one block each, its levels separated by
+// barriers instead of launches.  Measured on a GB300, a launch per level against
+// this: 1D Burgers L = 9 15.84 / 14.95 ms, L = 10 17.8 / 17.1, L = 12 10.99 /
+// 10.20; with as many cells in 2D (Euler L = 6) 6.08 / 6.06 and in 3D (Burgers
+// L = 4) 0.80 / 0.84 ms, whose nodes hold more work than one block has threads.
 constexpr int kOneBlockThreads = 256;
 constexpr long long kOneBlock = kOneBlockThreads * kStep;
 
@@ -393,10 +395,12 @@ static void adapt_dm(Launcher& L, int la, bool check)
     if (g.prec) pdl_launch(k_detail<D, M, float>, blocks_list(g, hi), NTHREADS, 0, L.st, g, la, hi);
     else pdl_launch(k_detail<D, M, double>, blocks_list(g, hi), NTHREADS, 0, L.st, g, la, hi);
     ++L.n;
-    if (g.N[g.L] <= kOneBlock) {
-        pdl_launch(k_flag_small<D>, 1, kOneBlockThreads, 0, L.st, g, la, check);
-        ++L.n;
-        return;
+    if constexpr (D == 1) {
+        if (g.N[g.L] <= kOneBlock) {
+            pdl_launch(k_flag_small<D>, 1, kOneBlockThreads, 0, L.st, g, la, check);
+            ++L.n;
+            return;
+        }
     }
     pdl_launch(k_mark<D>, blocks_step(g, hi), NTHREADS, 0, L.st, g, la, hi, la, check, check && la == hi);
     ++L.n;
@@ -409,11 +413,13 @@ template <int D, int M>
 static void apply_dm(Launcher& L, int la)
 {
     const Grid& g = L.g;
-    if (g.N[g.L] <= kOneBlock) {
-        if (g.prec) pdl_launch(k_install_small<D, M, float>, 1, kOneBlockThreads, 0, L.st, g, la);
-        else pdl_launch(k_install_small<D, M, double>, 1, kOneBlockThreads, 0, L.st, g, la);
-        ++L.n;
-        return;
+    if constexpr (D == 1) {
+        if (g.N[g.L] <= kOneBlock) {
+            if (g.prec) pdl_launch(k_install_small<D, M, float>, 1, kOneBlockThreads, 0, L.st, g, la);
+            else pdl_launch(k_install_small<D, M, double>, 1, kOneBlockThreads, 0, L.st, g, la);
+            ++L.n;
+            return;
+        }
     }
     const int b0 = blocks_list(g, g.L), b1 = blocks_step(g, la);
     if (g.prec) pdl_launch(k_release_apply<D, M, float>, b0 > b1 ? b0 : b1, NTHREADS, 0, L.st, g, la);
