@@ -220,7 +220,6 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
                                             unsigned char* smem)
 {
     const bool halt = halted(g); // with the loads below in one trip
-    const double dt = *g.dtp;    // fine step of the macro step
     using S = TileShape<EQ, D, R>;
     using Bits = typename Tile<D>::Bits;
     constexpr int M = S::M, TX = S::TX, TY = S::TY, TZ = S::TZ, NT = S::NT, H = S::H, NC = S::NC;
@@ -268,8 +267,6 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
     int u = lo, at = task;
     for (int c; at >= (c = g.counts[2 * (LMAX + 1) + u]); ++u) at -= c;
     const int tile = one && task == (int)blockIdx.x ? tile0 : g.tlist[g.toff[u] + at];
-    const double dtl = g.gts ? dt : ldexp(dt, g.L - u); // Eq. 13 step of level u
-    const double bw = dtl * bstage; // register weight dt_l b_s
     const int n = g.n[u];
     const int ntx = g.ntx[u], nty = g.nty[u];
     const int ox = (tile % ntx) * TX;
@@ -588,6 +585,12 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
         pdl_enter();
         waited = true;
     }
+    // the fine step is a value too: when the first stage of a macro step follows
+    // directly on the launch that sets it (a tree of one level only), nothing but
+    // this wait orders the two
+    const double dt = *g.dtp;
+    const double dtl = g.gts ? dt : ldexp(dt, g.L - u); // Eq. 13 step of level u
+    const double bw = dtl * bstage; // register weight dt_l b_s
     const int nst = sCount[0], nvc = sCount[1], nlf = sCount[2];
 
     // 3. one trip: exposures of stored and parent cells and of the finer-side
