@@ -2,6 +2,7 @@
 // layout, the LT iteration schedule (Alg. 3), the global-step MR iteration,
 // macro steps with the CFL rule, and read-back.
 #include "mrlt.h"
+#include "mrlt_input.h"
 #include "mrlt_macro.cuh"
 #include "mrlt_tree.cuh"
 
@@ -1021,22 +1022,24 @@ bool reads_host_memory()
     return known[dev].load() == 2;
 }
 
-// The caller's finest data into q^n of the finest nodes.  Large data are read in
-// place where kernels can: a copy from pageable memory goes through the driver's
-// staging buffers at the speed of one host thread, so that with data not in the
-// host's caches a 3D solve at L = 8 (671 MB of data, mixed, 32 iterations) took
-// 139 ms on a GB300 with the copy and 50 ms without; at 8 MB (2D, L = 9) both
-// ways take the same.  Not for memory that is released right after
-// (h->copy_input): unmapping what the GPU has read costs more than the copy (a
-// server mix of 12 requests 65 against 60 ms).  The caller's memory is read
-// until the stream has been waited for, before the call returns.
-constexpr size_t kReadInPlace = 16u << 20;
-
+// The caller's finest data into q^n of the finest nodes.  Large data on their
+// boundary are read in place where kernels can (read_in_place): a copy from
+// pageable memory goes through the driver's staging buffers at the speed of one
+// host thread.  Measured on a GB300, a fresh array per pass, reset and the
+// caller's own release of the array, in place / copied: 17 MB 0.53 / 0.57 ms,
+// 33 MB 1.04 / 1.11, 84 MB 1.97 / 2.17, 134 MB 3.05 / 3.30, 671 MB 11.3 / 11.8
+// (the release alone takes the same either way); with the host's caches flushed
+// before the call 0.64 / 0.69, 1.17 / 1.24, 2.09 / 2.20, 3.08 / 3.26 and 11.2 /
+// 11.8 ms.  At 8 MB both ways take 0.40 ms.  On a host whose staging was slow a 3D
+// solve at L = 8 (671 MB, 32 iterations) took 139 ms with the copy and 50 without.
+// A server's own vectors, released right after (h->copy_input), are copied: its
+// mix of 12 requests took 65 ms in place and 60 copied.  The caller's memory is
+// read until the stream has been waited for, before the call returns.
 mr_status load_finest(mr_solver* h, const double* q0)
 {
     Grid& g = h->K.g;
     const size_t bytes = (size_t)g.N[g.L] * g.m * sizeof(double);
-    if (bytes >= kReadInPlace && !h->copy_input && reads_host_memory()) {
+    if (read_in_place(q0, bytes, h->copy_input, reads_host_memory())) {
         h->K.store_finest(q0);
         return MR_OK;
     }
