@@ -433,10 +433,16 @@ __device__ __forceinline__ R minmod(R a, R b)
     if (a * b <= R(0)) return R(0);
     return fabs(a) < fabs(b) ? a : b;
 }
+// The same on the bit patterns.  A NaN leaves b, as in the comparisons above: a NaN
+// in b passes on to the slope.  (Differences hold quiet NaNs only, whose high word
+// lies above infinity's.)
 __device__ __forceinline__ double minmod(double a, double b)
 {
-    const double m = below_abs(a, b) ? a : b;
-    return (__double2hiint(a) ^ __double2hiint(b)) < 0 ? 0.0 : m;
+    const unsigned ha = (unsigned)__double2hiint(a) << 1, hb = (unsigned)__double2hiint(b) << 1;
+    const bool take_a = below_abs(a, b);
+    const double m = take_a ? a : b;
+    const double r = (__double2hiint(a) ^ __double2hiint(b)) < 0 ? 0.0 : m;
+    return (take_a ? hb : ha) > 0xffe00000u ? b : r;
 }
 
 // 1 / x and 1 / sqrt(x) in FP64 for the fluxes: the hardware's approximation
