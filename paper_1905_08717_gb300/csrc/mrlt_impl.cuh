@@ -445,28 +445,14 @@ __device__ __forceinline__ double minmod(double a, double b)
     return (take_a ? hb : ha) > 0xffe00000u ? b : r;
 }
 
-// 1 / x and 1 / sqrt(x) in FP64 for the fluxes: the hardware's approximation
-// (PTX rcp / rsqrt.approx.ftz.f64, some 20 bits) improved by one step of
-// Householder's method of third order.  With e = 1 - x y, or 1 - x y^2, the
-// exact results are y (1 + e + e^2 + ...) and y (1 + e/2 + 3 e^2/8 + ...), so the
-// terms left out are below 2^-54; the result is within one unit in the last
-// place, for 3 and 5 FP64 operations, where the general functions, which also
-// serve subnormals and infinities, take about twice that.  Zero gives a NaN.
-__device__ __forceinline__ double recip(double x)
-{
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-__device__ __forceinline__ float recip(float x) { return 1.0f / x; }
-__device__ __forceinline__ double recip_sqrt(double x)
-{
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-(x * y), y, 1.0);
-    return fma(y, e * fma(0.375, e, 0.5), y);
-}
+// 1 / x and 1 / sqrt(x) for the fluxes, correctly rounded and CUDA's rsqrt: over
+// all of FP64, subnormal densities and pressures included.  A third-order step
+// from the hardware's approximation, which takes 4% fewer FP64 operations in a
+// full-grid stage launch, loses both: it is good to one unit in the last place
+// only and gives a NaN for subnormals and infinities.
+template <class R>
+__device__ __forceinline__ R recip(R x) { return R(1) / x; }
+__device__ __forceinline__ double recip_sqrt(double x) { return rsqrt(x); }
 
 // a[k] for a run-time direction k < D: selects, where an indexed register
 // array would have to live in local memory
@@ -554,10 +540,9 @@ __device__ __forceinline__ void ausm_plus(R gam, int k, const R* PL, const R* PR
     F[D + 1] = a * (mp * (PL[0] * HL) + mm * (PR[0] * HR));
 }
 
-// The same in FP64 with fewer operations: three reciprocals instead of six divisions (a*^2
-// / a* = a* unless the normal flow is above critical; one reciprocal of the
-// interface speed), the polynomials of a side shared by its two splits, and
-// the flux from the two mass fluxes.
+// The same in FP64 with fewer operations: four divisions instead of six (a*^2
+// / a* = a* unless the normal flow is above critical), the polynomials of a side
+// shared by its two splits, and the flux from the two mass fluxes.
 __device__ __forceinline__ void ausm_split(double M, double sgn, double& mach, double& pres)
 {
     if (!below_abs(M, 1.0)) {
@@ -582,18 +567,19 @@ __device__ __forceinline__ void ausm_plus64(const Grid& g, int k, const double* 
         keR = fma(PR[1 + c], PR[1 + c], keR);
     }
     const double hp = g.igm + 1.0; // enthalpy of pressure: p g / (g - 1)
-    const double HL = fma(hp, pL * recip(PL[0]), 0.5 * keL), HR = fma(hp, pR * recip(PR[0]), 0.5 * keR);
+    const double HL = fma(hp, pL / PL[0], 0.5 * keL), HR = fma(hp, pR / PR[0], 0.5 * keR);
     const double uL = along<D>(PL + 1, k), uR = along<D>(PR + 1, k);
     const double cst = g.cstar; // 2 (g - 1) / (g + 1)
     const double aL2 = cst * HL, aR2 = cst * HR;
-    double aL = aL2 * recip_sqrt(aL2), aR = aR2 * recip_sqrt(aR2);
-    if (less(aL, uL)) aL = aL2 / uL;
-    if (less(aR, -uR)) aR = aR2 / -uR;
     // a side without a critical speed leaves the interface speed to the other
-    const double a = !positive(aL2) ? aR : (!positive(aR2) || less(aL, aR) ? aL : aR), ia = recip(a);
+    const bool okL = positive(aL2), okR = positive(aR2);
+    double aL = sqrt(aL2), aR = sqrt(aR2);
+    if (okL && less(aL, uL)) aL = aL2 / uL;
+    if (okR && less(aR, -uR)) aR = aR2 / -uR;
+    const double a = !okL ? aR : (!okR || less(aL, aR) ? aL : aR);
     double m1, p1, m2, p2;
-    ausm_split(uL * ia, 1.0, m1, p1);
-    ausm_split(uR * ia, -1.0, m2, p2);
+    ausm_split(uL / a, 1.0, m1, p1);
+    ausm_split(uR / a, -1.0, m2, p2);
     const double mh = a * (m1 + m2), ph = fma(p1, pL, p2 * pR);
     const bool back = negative(mh);
     const double fL = back ? 0.0 : mh * PL[0], fR = back ? mh * PR[0] : 0.0; // mass fluxes
@@ -605,16 +591,17 @@ __device__ __forceinline__ void ausm_plus64(const Grid& g, int k, const double* 
 
 // HLL in FP64 from the reconstructed primitives, by its weights: with
 // w_L = s_R / (s_R - s_L) and w_R = -s_L / (s_R - s_L) (1 and 0 when both waves
-// run one way) the flux is sum over the sides of w (F(U) - s U), s the
-// other... outer speed of that side, i.e. U (w (u_n - s)) plus w times the pressure terms.
-// The two mass fluxes rho w (u_n - s) carry momentum and kinetic energy, so
-// neither the conservative states nor the physical fluxes are formed.  Counted
-// by the hardware on a full grid (2D, all leaves): 214 FP64 operations per leaf
-// and stage, at 77% of the FP64 units' time.  Measured on a GB300 when this, the
+// run one way) the flux is w_L F(U_L) + w_R F(U_R) + d (U_R - U_L), d = s_L w_L =
+// -s_R w_R: each side gives U (w u_n -+ d), - on the left, plus w times the
+// pressure terms.  The two mass fluxes rho (w u_n -+ d) carry momentum and kinetic
+// energy, so neither the conservative states nor the physical fluxes are formed;
+// with one d for both sides its rounding cancels between like states (with
+// w (u_n - s) for each side, one operation more, the root mean square error of
+// the mass flux is 0.238 x 2^-53 of rho (|u| + c) against 0.195; rho, u and p of
+// order one, neighbours within 10%).  Measured on a GB300 when this, the
 // comparisons above and child() replaced the general forms, mean stage-2 launch:
 // 2D Euler L = 10 from 43.9 to 35.8 us on level 10 and 33.3 to 24.9 us on level
-// 9, 3D blast L = 7 from 308 to 243 us on level 7; recip, recip_sqrt and abs_bits
-// then took the full-grid launch (262 k leaves) from 155 to 133 us.
+// 9, 3D blast L = 7 from 308 to 243 us on level 7.
 template <int D, int M>
 __device__ __forceinline__ void hll64(const Grid& g, int k, const double* PL, const double* PR, double* F)
 {
@@ -633,7 +620,8 @@ __device__ __forceinline__ void hll64(const Grid& g, int k, const double* PL, co
     const bool allL = (okL || okR) && !negative(sL), allR = (okL || okR) && !allL && !positive(sR);
     const double ids = recip(sR - sL);
     double wL = sR * ids, wR = -sL * ids;
-    double aL = wL * (uL - sL), aR = wR * (uR - sR);
+    const double d = sL * wL;
+    double aL = fma(wL, uL, -d), aR = fma(wR, uR, d);
     if (allL || allR) {
         wL = allL ? 1.0 : 0.0;
         wR = allL ? 0.0 : 1.0;
