@@ -511,12 +511,12 @@ void stage(mr_solver* h, int lo, int hi, int s, int lmin)
         if (h->ev_used * 2 + 2 > (int)h->ev.size()) drain_events(h);
         cudaEventRecord(h->ev[2 * h->ev_used], h->stream);
         h->ev_level[h->ev_used] = hi;
-        launched = launch_stage(g, h->stream, lo, hi, s, lmin, b, reg);
+        launched = launch_stage(g, h->stream, lo, hi, s, lmin, b, reg, h->K.enter(), h->K.tick());
         cudaEventRecord(h->ev[2 * h->ev_used + 1], h->stream);
         ++h->ev_used;
         h->prof_launches += launched > 0 ? launched : 0;
     } else {
-        launched = launch_stage(g, h->stream, lo, hi, s, lmin, b, reg);
+        launched = launch_stage(g, h->stream, lo, hi, s, lmin, b, reg, h->K.enter(), h->K.tick());
     }
     if (launched < 0) {
         h->launch_failed = true;
@@ -596,15 +596,15 @@ mr_status lt_iteration(mr_solver* h, long long n, int part = 0)
     if (remesh) MR_TRY(adapt(h, lmin, part, mid));
     if (part == 1) return MR_OK;
     stage(h, lmin, L, 1, lmin); // first stage: all active levels at once
-    h->K.project_up(L - 1, lmin, PM_REF2, -1, true);
+    h->K.project_up(L - 1, lmin, PM_REF2);
     for (int l = L; l >= lmin; --l) {
-        if (l < L) h->K.project(l, PM_PRJ2, true);
+        if (l < L) h->K.project(l, PM_PRJ2);
         stage(h, l, l, 2, lmin);
     }
     if (g.rk == 3) {
-        h->K.project_up(L - 1, lmin, PM_REF3, -1, true);
+        h->K.project_up(L - 1, lmin, PM_REF3);
         for (int l = L; l >= lmin; --l) {
-            if (l < L) h->K.project(l, PM_PRJ3, true);
+            if (l < L) h->K.project(l, PM_PRJ3);
             stage(h, l, l, 3, lmin);
         }
     }
@@ -632,10 +632,10 @@ mr_status gts_iteration(mr_solver* h, long long n, int part = 0)
         MR_TRY(adapt(h, lb, part));
     if (part == 1) return MR_OK;
     stage(h, lb, L, 1, lb); // every level at the same instant: one launch per stage
-    h->K.project_up(L - 1, lb, PM_Q1, -1, true);
+    h->K.project_up(L - 1, lb, PM_Q1);
     stage(h, lb, L, 2, lb);
     if (g.rk == 3) {
-        h->K.project_up(L - 1, lb, PM_Q2, -1, true);
+        h->K.project_up(L - 1, lb, PM_Q2);
         stage(h, lb, L, 3, lb);
     }
     return MR_OK;
@@ -683,12 +683,14 @@ bool capture(mr_solver* h, Body body, cudaGraphExec_t* exec, long long* launches
         return false;
     }
     // stage-kernel attributes and occupancy are set up before capture begins
-    if (launch_stage(h->K.g, h->stream, 1, 0, 1, 0, 0.0, 0) < 0) return false;
+    if (launch_stage(h->K.g, h->stream, 1, 0, 1, 0, 0.0, 0, TreeSync{}, 0) < 0) return false;
     cudaStream_t user = h->stream;
     const long long k0 = h->K.n, s0 = h->stage_launches;
     h->stream = h->K.st = h->cap_stream;
     bool ok = cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+    h->K.piece_begin();
     const mr_status r = ok ? body() : MR_OK;
+    h->K.piece_end();
     cudaGraph_t graph = nullptr;
     if (ok) ok = cudaStreamEndCapture(h->cap_stream, &graph) == cudaSuccess && r == MR_OK && !h->launch_failed;
     h->stream = h->K.st = user;
@@ -716,8 +718,6 @@ bool capture(mr_solver* h, Body body, cudaGraphExec_t* exec, long long* launches
 // the host of a GB300, and every resize of the node arrays repeats them: a 1D
 // Burgers solve of two macro steps at L = 10, made from nothing, takes 28.4 ms
 // against 39.8 ms with its macro step of 256 iterations captured whole.
-constexpr long long kBlockIters = 16;
-
 long long block_iters(long long nit) { return nit < kBlockIters ? nit : kBlockIters; }
 
 bool capture_piece(mr_solver* h, mr_solver::Piece& x, long long reflux, long long n0, long long n1, long long nit)
@@ -749,6 +749,7 @@ mr_status run_macro(mr_solver* h, long long nit)
 {
     auto launch = [&](const mr_solver::Piece& x) -> mr_status {
         MR_CK(cudaGraphLaunch(x.exec, h->stream));
+        h->K.stale = true; // for the direct launches after it
         h->K.n += x.launches;
         h->stage_launches += x.stage_launches;
         return MR_OK;
@@ -778,6 +779,7 @@ mr_status head_enqueue(mr_solver* h)
     if (!h->prof && !h->graph_off) {
         if (h->head_exec || capture(h, body, &h->head_exec, &h->head_launches, nullptr)) {
             MR_CK(cudaGraphLaunch(h->head_exec, h->stream));
+            h->K.stale = true;
             h->K.n += h->head_launches;
             graphed = true;
         } else {
@@ -871,6 +873,7 @@ mr_status run_persistent(mr_solver* h, long long count, long long nit)
         return MR_E_CUDA;
     }
     ++h->K.n;
+    h->K.stale = true;
     h->wmax_valid = false;
     if (h->prof) MR_TRY(drain_stamps(h));
     return MR_OK;
@@ -1066,7 +1069,9 @@ mr_status fresh_state(mr_solver* h, const double* q0)
     MR_CK(cudaMemsetAsync(g.counts, 0, 3 * (LMAX + 1) * sizeof(int), h->stream));
     MR_CK(cudaMemsetAsync(g.err, 0, sizeof(int), h->stream));
     MR_CK(cudaMemsetAsync(g.room, 0, 5 * sizeof(int), h->stream));
-    MR_CK(cudaMemsetAsync(g.tick, 0, 2 * sizeof(int), h->stream));
+    MR_CK(cudaMemsetAsync(g.built, 0, kBuiltWords * sizeof(unsigned), h->stream));
+    h->K.published[1] = 0;
+    h->K.stale = true;
     MR_CK(cudaMemsetAsync(g.near, 0, sizeof(unsigned long long), h->stream));
     MR_CK(cudaMemsetAsync(g.updates, 0, sizeof(unsigned long long), h->stream));
     for (int l = g.lb; l <= g.L; ++l)
@@ -1158,7 +1163,7 @@ mr_status layout_alloc(mr_solver* h, const mr_config* cfg)
     A(dev_alloc(h, &g.tlist, (size_t)toff));
     A(dev_alloc(h, &g.scale_bits, MMAX));
     A(dev_alloc(h, &g.dtp, 1));
-    A(dev_alloc(h, &g.tick, 2));
+    A(dev_alloc(h, &g.built, kBuiltWords));
     A(dev_alloc(h, &g.room, 5));
     A(dev_alloc(h, &g.err, 1));
     A(dev_alloc(h, &g.near, 1));

@@ -72,7 +72,8 @@ struct Grid {
     unsigned long long* wmax;
     unsigned long long* updates;
     unsigned long long* work;       // [(LMAX+1) * 4]: leaf-stages per level and stage
-    int* tick;                      // [2] tile tickets of stage launches, by parity of the stage
+    unsigned* built;                // [0] publications of the running captured piece, [1] of direct launches (see
+                                    // TreeSync); tile tickets: [2] of direct stage launches, [3..] of the piece's
     double* dtp;                    // fine step dt of the current macro step (device scalar)
     int* room;                      // [0] refinement flags being counted, [1] halt: iteration + 1, [2] nodes needed,
                                     // [3] blocks that counted, [4] iteration of the macro step
@@ -95,12 +96,13 @@ struct Grid {
     int gcap;                       // CTAs per stage launch at most (0: resident capacity)
 };
 
-// Programmatic dependent launch (sm_90 and later).  Every kernel starts by
-// waiting until the kernel before it in the stream has completed and its
-// writes are visible (griddepcontrol.wait), then allows the next kernel's
-// launch to begin (griddepcontrol.launch_dependents).  The launch and the CTA
-// setup of the next kernel thus overlap the tail of this one.  Both are no-ops
-// in a kernel launched without a programmatic dependency.
+// Programmatic dependent launch (sm_90 and later).  Every thread of every kernel
+// waits until the kernel before it in the stream has completed and its writes are
+// visible (griddepcontrol.wait), then allows the next kernel's launch to begin
+// (griddepcontrol.launch_dependents).  The launch and the CTA setup of the next
+// kernel thus overlap the tail of this one.  Most kernels wait first; those that
+// leave the tree alone may look it up before (tree_enter).  Both are no-ops in a
+// kernel launched without a programmatic dependency.
 __device__ __forceinline__ void pdl_enter()
 {
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -111,8 +113,57 @@ __device__ __forceinline__ void pdl_enter()
 // the arrays hold halts the solver's device work (room[1] != 0): every later
 // kernel of the fine iterations returns at its start, until the host has
 // grown the arrays, cleared the halt and resumed at the halted iteration.
-// Read after pdl_enter, so that a halt set by an earlier kernel is visible.
+// Read after pdl_enter, or after tree_enter: the remesh that sets it comes before
+// the publication that follows the remesh.
 __device__ __forceinline__ bool halted(const Grid& g) { return g.room[1] != 0; }
+
+// Lookups before the wait: the tree (counts, lists, statuses, slots), the halt
+// and the fine step.  A kernel's own wait makes its predecessor's writes visible;
+// those of the launches before that one have to be known to be visible in another
+// way, which TreeSync holds for each launch of a kernel that leaves the tree alone:
+//  - kVisible: captured in a piece of a macro step, with no remesh before it in
+//    the piece.  A graph launch is ordered with the stream, so a piece starts
+//    after everything before it.
+//  - kPublish: the first kernel after a remesh, or after anything else of the
+//    kind.  It waits first, and then adds one to g.built[word] with release order.
+//  - kAcquire: it reads g.built[word] with acquire order, and a count of at least
+//    `need` shows that the last publication before it, and with it all that is
+//    looked up, is visible; otherwise it waits first.  No older value can be
+//    taken for that count: word 0, of captured launches, counts within a piece and
+//    is cleared at the end of each (k_piece_end); word 1, of direct launches, only
+//    grows, and the host knows the count.
+// tree_enter is called by every thread of the CTA and returns whether this one has
+// waited.  Measured on a GB300 against waiting first everywhere: 1D Burgers L = 10
+// 17.9 / 20.9 ms, 2D Burgers L = 10 83.5 / 95.3, global step L = 9 72.0 / 77.1, 3D
+// blast L = 7 35.6 / 39.1, 2D Euler L = 10 opening, FP64 179 / 204 and mixed 73.7 /
+// 85.3 ms.  In 2D and 3D one thread reads the count for its CTA (with a read by
+// every warp 2D Burgers took 1% and 2D Euler 1.5% longer); the small CTAs of 1D
+// read it with every thread (one thread and a barrier: 2% longer).
+enum TreeMode { kVisible = 0, kAcquire, kPublish };
+struct TreeSync {
+    int mode, word;
+    unsigned need;
+};
+template <int D>
+__device__ __forceinline__ bool tree_enter(const Grid& g, const TreeSync& t)
+{
+    if (t.mode == kVisible) return false;
+    if (t.mode == kAcquire) {
+        unsigned n = t.need - 1;
+        if (D == 1 || threadIdx.x == 0)
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(g.built + t.word) : "memory");
+        const bool there = (int)(n - t.need) >= 0;
+        if (D == 1 ? there : __syncthreads_or(there) != 0) return false;
+    } else {
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (blockIdx.x == 0) { // before this CTA lets the next kernel start
+            if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(g.built + t.word) : "memory");
+            __syncthreads();
+        }
+    }
+    pdl_enter();
+    return true;
+}
 
 #define MRLT_ENTER(g)         \
     do {                      \
@@ -758,7 +809,14 @@ struct Launch; // fwd
 // levels only), fine step dt = *g.dtp (level u steps dt, or 2^{L-u} dt in LT
 // mode), RK weight b of the stage; returns the number of kernel launches issued
 // (-1 when the kernel could not be set up).  lo > hi only sets the kernel up.
-int launch_stage(const Grid& g, cudaStream_t st, int lo, int hi, int s, int lmin, double b, int reg);
+// sync: see TreeSync; tick: the index of its tile tickets in g.built.
+int launch_stage(const Grid& g, cudaStream_t st, int lo, int hi, int s, int lmin, double b, int reg, TreeSync sync,
+                 int tick);
+// words of g.built: three, and one for each stage launch of a captured piece (at
+// most kBlockIters iterations of one launch and two for each level)
+constexpr int kBlockIters = 16;
+constexpr int kDirectTick = 2, kFirstTick = 3;
+constexpr int kBuiltWords = kFirstTick + kBlockIters * (1 + 2 * (LMAX + 1));
 void launch_wave(const Grid& g, cudaStream_t st);
 // one persistent macro-step kernel launch (mrlt_macro.cuh); a == nullptr sets
 // the kernel up only.  Returns 1 when launched, 0 after set-up, -1 on failure.

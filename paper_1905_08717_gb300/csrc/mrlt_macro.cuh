@@ -117,7 +117,7 @@ template <int EQ, int D, class R>
 __device__ __noinline__ void mph_stage(const Grid& g, int lo, int hi, int s, int lmin, double b, int reg,
                                        unsigned char* smem)
 {
-    stage_tiles<EQ, D, R, false>(g, lo, hi, s, lmin, b, reg, smem);
+    stage_tiles<EQ, D, R, false>(g, lo, hi, s, lmin, b, reg, TreeSync{}, 0, smem);
 }
 template <int D, int M, class T>
 __device__ __noinline__ void mph_project(const Grid& g, int l, int mode)

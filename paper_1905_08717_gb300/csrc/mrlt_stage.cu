@@ -13,13 +13,14 @@ __global__ void __launch_bounds__(NTHREADS) k_wave(const __grid_constant__ Grid 
     dev_wave<EQ, D, T>(g, g.lb, g.L);
 }
 
-int launch_stage(const Grid& g, cudaStream_t st, int lo, int hi, int s, int lmin, double b, int reg)
+int launch_stage(const Grid& g, cudaStream_t st, int lo, int hi, int s, int lmin, double b, int reg, TreeSync sync,
+                 int tick)
 {
     switch (g.eq) {
-    case 0: return launch_stage_eq<0>(g, st, lo, hi, s, lmin, b, reg);
-    case 1: return launch_stage_eq<1>(g, st, lo, hi, s, lmin, b, reg);
-    case 2: return launch_stage_eq<2>(g, st, lo, hi, s, lmin, b, reg);
-    case 3: return launch_stage_eq<3>(g, st, lo, hi, s, lmin, b, reg);
+    case 0: return launch_stage_eq<0>(g, st, lo, hi, s, lmin, b, reg, sync, tick);
+    case 1: return launch_stage_eq<1>(g, st, lo, hi, s, lmin, b, reg, sync, tick);
+    case 2: return launch_stage_eq<2>(g, st, lo, hi, s, lmin, b, reg, sync, tick);
+    case 3: return launch_stage_eq<3>(g, st, lo, hi, s, lmin, b, reg, sync, tick);
     default: return 0;
     }
 }

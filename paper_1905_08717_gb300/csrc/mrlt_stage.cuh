@@ -203,23 +203,25 @@ __device__ __noinline__ void far_value(const Grid& g, Ctx x, int l, int p0, int 
 // is the dynamic shared memory of TileShape::SMEM bytes.  Called by
 // k_stage_tile and by the persistent macro-step kernel.
 //
-// EARLY (k_stage_tile): phases 1 and 2 read nothing but the tree, and no
-// kernel that changes the tree comes directly before a stage launch.  So they
-// run before the wait for that kernel's results (pdl_enter): when this launch
-// starts, every CTA of its predecessor has itself waited for its own, so
-// whatever built the tree is complete.  The first tile's status trips, masks and
-// lookups thus overlap the predecessor.  CTAs that start early land on SMs
-// unevenly, so a launch with more tiles than CTAs hands out those after every
-// CTA's first by a counter, in the order the CTAs ask (tiles fixed to CTAs made
-// an early start 10% slower).  The CTA that takes the last ticket clears the
-// counter.  Two counters by the parity of the stage: the
-// launch before the last that uses the same one is complete when this one
-// starts.
+// EARLY (k_stage_tile): phases 1 and 2 read nothing but the tree, so they run
+// before the wait for the predecessor's results where the tree is visible by
+// then (tree_enter).  The first tile's status trips, masks and lookups thus
+// overlap the predecessor.  CTAs that start early land on SMs unevenly, so a
+// launch with more tiles than CTAs hands out those after every CTA's first by a
+// counter, in the order the CTAs ask (tiles fixed to CTAs made an early start 10%
+// slower).  Every launch of a captured piece has a counter of its own, 0 since
+// before the piece, and asks before the wait; direct launches share one, ask
+// after the wait, and the CTA that takes the last ticket clears it for the next.
 template <int EQ, int D, class R, bool EARLY>
 __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s, int lmin, double bstage, int reg,
-                                            unsigned char* smem)
+                                            const TreeSync& sync, int tick, unsigned char* smem)
 {
+    bool waited = !EARLY || tree_enter<D>(g, sync);
     const bool halt = halted(g); // with the loads below in one trip
+    // the fine step, set by a launch of its own before the macro step's pieces;
+    // direct launches publish it like a tree (on a tree of one level a stage may
+    // follow directly on the launch that sets the step)
+    const double dt = *g.dtp;
     using S = TileShape<EQ, D, R>;
     using Bits = typename Tile<D>::Bits;
     constexpr int M = S::M, TX = S::TX, TY = S::TY, TZ = S::TZ, NT = S::NT, H = S::H, NC = S::NC;
@@ -260,7 +262,6 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
     const bool one = lo == hi && (int)blockIdx.x < g.ntx[lo] * g.nty[lo] * g.ntz[lo];
     const int tile0 = one ? g.tlist[g.toff[lo] + blockIdx.x] : 0;
     if (halt) ntask = 0;
-    bool waited = !EARLY;
     const bool handed = EARLY && ntask > (int)gridDim.x; // tiles beyond the first by tickets
     __shared__ int sNext;
     for (int task = blockIdx.x; task < ntask;) {
@@ -320,11 +321,7 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
     if (tid < PBY * PBZ) sPar[tid] = 0;
     if (tid == 0) sWord[0][NW] = sWord[1][NW] = 0;
     __syncthreads();
-    if (handed && tid == 0) {
-        const int ticket = atomicAdd(&g.tick[s & 1], 1);
-        if (ticket == ntask - 1) g.tick[s & 1] = 0;
-        sNext = (int)gridDim.x + ticket;
-    }
+    if (handed && tid == 0 && tick != kDirectTick) sNext = (int)(gridDim.x + atomicAdd(&g.built[tick], 1u));
 
     // 2. row masks.  row(k, by, bz): the leaves (k = 0) or internal nodes (1)
     // of a row of the block, empty past it; tile_row: the tile's leaves in it
@@ -585,10 +582,11 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
         pdl_enter();
         waited = true;
     }
-    // the fine step is a value too: when the first stage of a macro step follows
-    // directly on the launch that sets it (a tree of one level only), nothing but
-    // this wait orders the two
-    const double dt = *g.dtp;
+    if (handed && tid == 0 && tick == kDirectTick) {
+        const int ticket = (int)atomicAdd(&g.built[tick], 1u);
+        if (ticket == ntask - 1) g.built[tick] = 0;
+        sNext = (int)gridDim.x + ticket;
+    }
     const double dtl = g.gts ? dt : ldexp(dt, g.L - u); // Eq. 13 step of level u
     const double bw = dtl * bstage; // register weight dt_l b_s
     const int nst = sCount[0], nvc = sCount[1], nlf = sCount[2];
@@ -929,10 +927,11 @@ __device__ __forceinline__ void stage_tiles(const Grid& g, int lo, int hi, int s
 
 template <int EQ, int D, class R>
 __global__ void __launch_bounds__(Tile<D>::THREADS, TileShape<EQ, D, R>::PERSM)
-k_stage_tile(const __grid_constant__ Grid g, int lo, int hi, int s, int lmin, double bstage, int reg)
+k_stage_tile(const __grid_constant__ Grid g, int lo, int hi, int s, int lmin, double bstage, int reg, TreeSync sync,
+             int tick)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    stage_tiles<EQ, D, R, true>(g, lo, hi, s, lmin, bstage, reg, smem);
+    stage_tiles<EQ, D, R, true>(g, lo, hi, s, lmin, bstage, reg, sync, tick, smem);
 }
 
 static inline int grid_for(const Grid& g, int l)
@@ -948,7 +947,8 @@ static inline int grid_for(const Grid& g, int l)
 // thread, so the result does not depend on the grid size or on which CTA
 // takes a tile.
 template <int EQ, int D, class R>
-static int stage_dispatch(const Grid& g, cudaStream_t st, int lo, int hi, int s, int lmin, double b, int reg)
+static int stage_dispatch(const Grid& g, cudaStream_t st, int lo, int hi, int s, int lmin, double b, int reg, TreeSync sync,
+                          int tick)
 {
     using S = TileShape<EQ, D, R>;
     constexpr int kMaxDev = 64;
@@ -972,7 +972,8 @@ static int stage_dispatch(const Grid& g, cudaStream_t st, int lo, int hi, int s,
     long long grid = total < resident[dev] ? total : resident[dev];
     if (g.gcap > 0 && grid > g.gcap) grid = g.gcap;
     if (grid < 1) grid = 1;
-    if (pdl_launch(k_stage_tile<EQ, D, R>, dim3((unsigned)grid), dim3(S::NT), S::SMEM, st, g, lo, hi, s, lmin, b, reg) !=
+    if (pdl_launch(k_stage_tile<EQ, D, R>, dim3((unsigned)grid), dim3(S::NT), S::SMEM, st, g, lo, hi, s, lmin, b, reg,
+                   sync, tick) !=
         cudaSuccess)
         return -1;
     return 1;
@@ -981,10 +982,11 @@ static int stage_dispatch(const Grid& g, cudaStream_t st, int lo, int hi, int s,
 // stage launcher of one equation (all dimensions, both precisions); each is
 // defined in its own translation unit so that they compile in parallel
 template <int EQ>
-int launch_stage_eq(const Grid& g, cudaStream_t st, int lo, int hi, int s, int lmin, double b, int reg);
-template <> int launch_stage_eq<0>(const Grid&, cudaStream_t, int, int, int, int, double, int);
-template <> int launch_stage_eq<1>(const Grid&, cudaStream_t, int, int, int, int, double, int);
-template <> int launch_stage_eq<2>(const Grid&, cudaStream_t, int, int, int, int, double, int);
-template <> int launch_stage_eq<3>(const Grid&, cudaStream_t, int, int, int, int, double, int);
+int launch_stage_eq(const Grid& g, cudaStream_t st, int lo, int hi, int s, int lmin, double b, int reg, TreeSync sync,
+                    int tick);
+template <> int launch_stage_eq<0>(const Grid&, cudaStream_t, int, int, int, int, double, int, TreeSync, int);
+template <> int launch_stage_eq<1>(const Grid&, cudaStream_t, int, int, int, int, double, int, TreeSync, int);
+template <> int launch_stage_eq<2>(const Grid&, cudaStream_t, int, int, int, int, double, int, TreeSync, int);
+template <> int launch_stage_eq<3>(const Grid&, cudaStream_t, int, int, int, int, double, int, TreeSync, int);
 
 } // namespace mrlt

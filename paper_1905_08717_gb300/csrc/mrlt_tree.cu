@@ -27,8 +27,8 @@ static inline int blocks_list(const Grid& g, int l)
 
 // ------------------------------------------------------------ kernels
 // Each kernel waits for its predecessor (programmatic dependent launch) and
-// runs one device body of mrlt_tree_dev.cuh over its own grid; kernels whose
-// predecessor leaves the tree alone look it up before they wait.  Most launches
+// runs one device body of mrlt_tree_dev.cuh over its own grid; kernels that leave
+// the tree alone look it up before they wait (tree_enter).  Most launches
 // are short chains of dependent trips, so that takes two or three of five trips
 // off them.  Measured on a GB300 with the stage kernel's early start, whole
 // solves: 1D Burgers L = 10 30.5 to 23.6 ms (made from nothing), 2D Burgers
@@ -42,19 +42,17 @@ __global__ void k_leaf_copy(const __grid_constant__ Grid g, int lo, int hi, int 
     dev_leaf_copy<M, T>(g, lo, hi, from, to);
 }
 
-// Up-sweep of levels hi..lo (one level: hi = lo); early as in kernel_list.
+// Up-sweep of levels hi..lo (one level: hi = lo).
 template <int D, int M, class T>
-__global__ void k_project_up(const __grid_constant__ Grid g, int hi, int lo, int mode, int top, bool early)
+__global__ void k_project_up(const __grid_constant__ Grid g, int hi, int lo, int mode, int top, TreeSync sync)
 {
-    if (!early) pdl_enter();
+    const bool waited = tree_enter<D>(g, sync);
     const int steps = up_steps(g, hi, lo);
-    for (int c = blockIdx.x; c < steps || early; c += gridDim.x) { // uniform across the CTA
-        const UpRefs<D> r = up_lookup<D>(g, hi, lo, c);
-        if (early) {
-            pdl_enter();
-            early = false;
-        }
-        if (halted(g)) return;
+    UpRefs<D> r = up_lookup<D>(g, hi, lo, blockIdx.x);
+    if (!waited) pdl_enter();
+    if (halted(g)) return;
+    for (int c = blockIdx.x; c < steps; c += gridDim.x) { // uniform across the CTA
+        if (c != (int)blockIdx.x) r = up_lookup<D>(g, hi, lo, c);
         up_project<D, M, T>(g, r, hi - lo, mode, top);
     }
 }
@@ -62,16 +60,16 @@ __global__ void k_project_up(const __grid_constant__ Grid g, int hi, int lo, int
 // The beginning of an iteration: q^n := end value of the leaves of levels
 // lo..L and, beside it, the up-sweep of levels uhi..ulo (which reads leaf
 // children's end values; ulo with mode top): one launch where the copy and the
-// sweep were two.  The tree is looked up before the wait, as in kernel_list: an
-// iteration's predecessor never changes the tree.
+// sweep were two.
 template <int D, int M, class T>
-__global__ void k_begin(const __grid_constant__ Grid g, int lo, bool next, int uhi, int ulo, int top)
+__global__ void k_begin(const __grid_constant__ Grid g, int lo, bool next, int uhi, int ulo, int top, TreeSync sync)
 {
+    const bool waited = tree_enter<D>(g, sync);
     const int steps = uhi >= ulo ? up_steps(g, uhi, ulo) : 0;
     UpRefs<D> r;
     if (uhi >= ulo) r = up_lookup<D>(g, uhi, ulo, blockIdx.x);
     kernel_list<0>(
-        g, lo, g.L, true, [&](int l, long long id) { return slot_of(g, l, id); },
+        g, lo, g.L, waited, [&](int l, long long id) { return slot_of(g, l, id); },
         [&](int sl) {
             T q[M];
             load_row<M, T>(nd<T>(g, F_QE, sl), q);
@@ -86,10 +84,10 @@ __global__ void k_begin(const __grid_constant__ Grid g, int lo, bool next, int u
 }
 
 template <int D, int M, class T>
-__global__ void k_detail(const __grid_constant__ Grid g, int lo, int hi)
+__global__ void k_detail(const __grid_constant__ Grid g, int lo, int hi, TreeSync sync)
 {
     kernel_list<1>(
-        g, lo, hi, true, [&](int l, long long id) { return lookup_detail<D>(g, l, id); },
+        g, lo, hi, tree_enter<D>(g, sync), [&](int l, long long id) { return lookup_detail<D>(g, l, id); },
         [&](const DetailRefs<D>& e) { detail_node<D, M, T>(g, e); });
 }
 
@@ -181,10 +179,10 @@ __global__ void k_cmp_scatter(const __grid_constant__ Grid g, LevelChunks lc, co
 }
 
 template <int D, int M, class T>
-__global__ void k_reflux(const __grid_constant__ Grid g, int lo, int hi)
+__global__ void k_reflux(const __grid_constant__ Grid g, int lo, int hi, TreeSync sync)
 {
     kernel_list<0>(
-        g, lo, hi, true, [&](int l, long long id) { return lookup_reflux<D>(g, l, id); },
+        g, lo, hi, tree_enter<D>(g, sync), [&](int l, long long id) { return lookup_reflux<D>(g, l, id); },
         [&](const RefluxRefs<D>& e) { reflux_leaf<D, M, T>(g, e); });
 }
 
@@ -345,24 +343,23 @@ static int up_blocks(const Grid& g, int ghi, int glo)
 }
 
 template <int D, int M>
-static void project_up_dm(Launcher& L, int hi, int lo, int mode, int top, bool early)
+static void project_up_dm(Launcher& L, int hi, int lo, int mode, int top)
 {
     static_assert((1 << (D * kUpDepth<D>)) * 2 <= NTHREADS, "two top nodes per CTA");
     for (int ghi = hi; ghi >= lo;) {
         const int glo = ghi - kUpDepth<D> > lo ? ghi - kUpDepth<D> : lo;
-        MRLT_T_LAUNCH(L, up_blocks(L.g, ghi, glo), (L.g, ghi, glo, mode, glo == lo ? top : mode, early),
+        MRLT_T_LAUNCH(L, up_blocks(L.g, ghi, glo), (L.g, ghi, glo, mode, glo == lo ? top : mode, L.enter()),
                       k_project_up<D, M);
         ++L.n;
         ghi = glo - 1;
-        early = true; // a sweep changes no tree
     }
 }
 
-void Launcher::project(int l, int mode, bool early) { MRLT_DM_DISPATCH(project_up_dm, *this, l, l, mode, mode, early); }
+void Launcher::project(int l, int mode) { MRLT_DM_DISPATCH(project_up_dm, *this, l, l, mode, mode); }
 
-void Launcher::project_up(int hi, int lo, int mode, int top, bool early)
+void Launcher::project_up(int hi, int lo, int mode, int top)
 {
-    if (hi >= lo) MRLT_DM_DISPATCH(project_up_dm, *this, hi, lo, mode, top < 0 ? mode : top, early);
+    if (hi >= lo) MRLT_DM_DISPATCH(project_up_dm, *this, hi, lo, mode, top < 0 ? mode : top);
 }
 
 template <int D, int M>
@@ -371,9 +368,10 @@ static void begin_dm(Launcher& L, int lmin, bool next, int lo, int top)
     const Grid& g = L.g;
     const int ghi = g.L - 1, glo = ghi - kUpDepth<D> > lo ? ghi - kUpDepth<D> : lo;
     const int b0 = blocks_list(g, g.L), b1 = ghi >= lo ? up_blocks(g, ghi, glo) : 1;
-    MRLT_T_LAUNCH(L, b0 > b1 ? b0 : b1, (g, lmin, next, ghi, glo, glo == lo ? top : (int)PM_BEG), k_begin<D, M);
+    MRLT_T_LAUNCH(L, b0 > b1 ? b0 : b1, (g, lmin, next, ghi, glo, glo == lo ? top : (int)PM_BEG, L.enter()),
+                  k_begin<D, M);
     ++L.n;
-    if (glo > lo) project_up_dm<D, M>(L, glo - 1, lo, PM_BEG, top, true);
+    if (glo > lo) project_up_dm<D, M>(L, glo - 1, lo, PM_BEG, top);
 }
 
 void Launcher::begin(int lmin, bool next, int lo, int top) { MRLT_DM_DISPATCH(begin_dm, *this, lmin, next, lo, top); }
@@ -392,8 +390,7 @@ static void adapt_dm(Launcher& L, int la, bool check)
 {
     const Grid& g = L.g;
     const int hi = g.L - 1; // levels whose nodes may own children
-    if (g.prec) pdl_launch(k_detail<D, M, float>, blocks_list(g, hi), NTHREADS, 0, L.st, g, la, hi);
-    else pdl_launch(k_detail<D, M, double>, blocks_list(g, hi), NTHREADS, 0, L.st, g, la, hi);
+    MRLT_T_LAUNCH(L, blocks_list(g, hi), (g, la, hi, L.enter()), k_detail<D, M);
     ++L.n;
     if constexpr (D == 1) {
         if (g.N[g.L] <= kOneBlock) {
@@ -441,12 +438,13 @@ void Launcher::compact(int lo, int hi)
     pdl_launch(k_cmp_count, total, NTHREADS, 0, st, g, lc, bc);
     pdl_launch(k_cmp_scatter, total + hi - lo + 1, NTHREADS, 0, st, g, lc, (const int*)bc);
     n += 2;
+    stale = true;
 }
 
 template <int D, int M>
 static void reflux_dm(Launcher& L, int lo, int hi)
 {
-    MRLT_T_LAUNCH(L, blocks_list(L.g, hi), (L.g, lo, hi), k_reflux<D, M);
+    MRLT_T_LAUNCH(L, blocks_list(L.g, hi), (L.g, lo, hi, L.enter()), k_reflux<D, M);
     ++L.n;
 }
 
@@ -622,6 +620,7 @@ void Launcher::renumber(const Grid& from, const int* counts_host, long long used
     long long cnt = used > g.cap - 1 - used ? used : g.cap - 1 - used;
     if (g.prec) pdl_launch(k_renumber<float>, blocks_dense(cnt), NTHREADS, 0, st, g, from, base, used);
     else pdl_launch(k_renumber<double>, blocks_dense(cnt), NTHREADS, 0, st, g, from, base, used);
+    stale = true;
     ++n;
 }
 
@@ -631,9 +630,36 @@ void Launcher::scale_init()
     ++n;
 }
 
+// the words of g.built that a captured piece used, after all its kernels
+__global__ void k_piece_end(const __grid_constant__ Grid g, int stages)
+{
+    pdl_enter(); // each kernel of the piece waited for the one before it
+    if (threadIdx.x == 0) g.built[0] = 0;
+    for (int i = threadIdx.x; i < stages; i += blockDim.x) g.built[kFirstTick + i] = 0;
+}
+
+void Launcher::piece_begin()
+{
+    capturing = true;
+    stale = false;
+    published[0] = 0;
+    stages = 0;
+}
+
+void Launcher::piece_end()
+{
+    if (published[0] || stages) {
+        pdl_launch(k_piece_end, 1, NTHREADS, 0, st, g, stages);
+        ++n;
+    }
+    capturing = false;
+    stale = true;
+}
+
 void Launcher::set_dt(double dt)
 {
     pdl_launch(k_set_dt, 1, 32, 0, st, g, dt);
+    stale = true;
     ++n;
 }
 

@@ -11,11 +11,29 @@ struct Launcher {
     cudaStream_t st = nullptr;
     int* bc = nullptr; // compaction scratch, 2 ints per block over all levels
     long long n = 0;   // kernel launches issued
+    // what the next kernel can rely on (see TreeSync)
+    bool capturing = false;
+    unsigned published[2] = {0, 0}; // publications, of the piece being captured and of direct launches
+    bool stale = true;              // something to look up has changed since the last publication
+    int stages = 0;                 // stage launches of the piece
 
-    // early: the kernel launched before does not change the tree (see kernel_list)
-    void project(int l, int mode, bool early = false);
+    // how the next kernel that looks the tree up enters
+    TreeSync enter()
+    {
+        const int word = capturing ? 0 : 1;
+        if (!stale) return {capturing && !published[0] ? kVisible : kAcquire, word, published[word]};
+        stale = false;
+        return {kPublish, word, ++published[word]};
+    }
+    // the index of a stage launch's tile tickets in g.built
+    int tick() { return capturing ? kFirstTick + stages++ : kDirectTick; }
+    // a captured piece begins; ends, with the words of g.built that it used cleared
+    void piece_begin();
+    void piece_end();
+
+    void project(int l, int mode);
     // levels hi..lo in fewer launches; level lo with mode top (mode if top < 0)
-    void project_up(int hi, int lo, int mode, int top = -1, bool early = false);
+    void project_up(int hi, int lo, int mode, int top = -1);
     // an iteration begins: leaf copy of levels lmin..L, up-sweep of levels L-1..lo
     // (level lo with mode top); next: it is not the macro step's first
     void begin(int lmin, bool next, int lo, int top);

@@ -67,19 +67,13 @@ __device__ __forceinline__ void for_list(const Grid& g, int lo, int hi, F f)
 }
 
 // for_list for a kernel's whole body, with the tree's share of an entry's work,
-// lookup(l, id), apart from the use(entry) of its result.  early: no kernel
-// that changes the tree directly precedes this launch, so the first entries are
-// looked up before the wait for the predecessor's values (pdl_enter): when this
-// kernel starts, each CTA of its predecessor has itself waited for its own, so
-// whatever built the tree is complete.  Otherwise the wait comes first.
+// lookup(l, id), apart from the use(entry) of its result: the first entries are
+// looked up before the wait for the predecessor's values where the tree is
+// visible by then (waited: what tree_enter returned).
 template <int KIND, class Lookup, class Use>
-__device__ __forceinline__ void kernel_list(const Grid& g, int lo, int hi, bool early, Lookup lookup, Use use)
+__device__ __forceinline__ void kernel_list(const Grid& g, int lo, int hi, bool waited, Lookup lookup, Use use)
 {
-    if (!early) {
-        pdl_enter();
-        if (halted(g)) return;
-    }
-    bool waited = !early, stop = false;
+    bool stop = waited && halted(g);
     const auto enter = [&]() {
         if (waited) return;
         pdl_enter();

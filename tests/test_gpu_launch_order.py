@@ -40,3 +40,45 @@ def test_one_level_tree_takes_the_step_of_its_macro_step(rk, prec):
         assert np.array_equal(va, vb), k
     a.close()
     b.close()
+
+
+def _problem(dim, eq, L, lb, mode, rk):
+    if eq == I.EQ_EULER:
+        p, q = (I.euler_2d_quadrants if dim == 2 else I.euler_3d_blast)(L=L, min_level=lb)
+    else:
+        p = I.Problem(dim=dim, equation=I.EQ_BURGERS, max_level=L, min_level=lb, eps=1e-2)
+        x = (np.arange(1 << L) + 0.5) / (1 << L)
+        g = np.meshgrid(*([x] * dim), indexing="ij")
+        q = sum(np.sin(2 * np.pi * (k + 1) * a + k) for k, a in enumerate(g))[None] * 0.5
+    return p.replace(time_mode=mode, rk_order=rk), np.ascontiguousarray(q)
+
+
+@pytest.mark.parametrize("dim,eq,L,lb,mode,rk", [
+    (1, I.EQ_BURGERS, 10, 2, I.TIME_LT, 3), (1, I.EQ_BURGERS, 14, 8, I.TIME_LT, 2), (1, I.EQ_BURGERS, 9, 4, I.TIME_GTS, 3),
+    (2, I.EQ_BURGERS, 8, 3, I.TIME_LT, 2), (2, I.EQ_EULER, 9, 4, I.TIME_LT, 3), (2, I.EQ_EULER, 8, 5, I.TIME_GTS, 2),
+    (3, I.EQ_EULER, 6, 3, I.TIME_LT, 3),
+])
+def test_direct_launches_equal_replayed_pieces(dim, eq, L, lb, mode, rk):
+    """whole macro steps from captured pieces (a), single iterations and mixed
+    counts launched directly between them (b), everything directly (c): the
+    publications of both kinds of launches interleave in b"""
+    import paper_1905_08717_gb300 as pkg
+    p, q = _problem(dim, eq, L, lb, mode, rk)
+    nit = 1 << (L - lb)
+    dt = 0.2 / (1 << L) / (12.0 if dim == 3 else 4.0)
+    a, b, c = (pkg.Solver(p, q) for _ in range(3))
+    c.profile(True)
+    for k in range(3):
+        a.iterate(dt, nit)
+        c.iterate(dt, nit)
+        if k == 1:
+            b.iterate(dt, nit)
+        else:
+            for n in (1, nit // 2, nit - 1 - nit // 2):
+                if n:
+                    b.iterate(dt, n)
+    (ka, va), (kb, vb), (kc, vc) = a.leaves(), b.leaves(), c.leaves()
+    assert np.array_equal(ka, kb) and np.array_equal(ka, kc)
+    assert np.array_equal(va, vb) and np.array_equal(va, vc)
+    for s in (a, b, c):
+        s.close()
