@@ -138,19 +138,20 @@ __global__ void k_release_apply(const __grid_constant__ Grid g, int la)
 // this: 1D Burgers L = 9 15.84 / 14.95 ms, L = 10 17.8 / 17.1, L = 12 10.99 /
 // 10.20; with as many cells in 2D (Euler L = 6) 6.08 / 6.06 and in 3D (Burgers
 // L = 4) 0.80 / 0.84 ms, whose nodes hold more work than one block has threads.
+// Whether the new tree fits is not asked: at most 8191 nodes of at most 244 bytes
+// always have a slot for every cell (kDenseBytes).
 constexpr int kOneBlockThreads = 256;
 constexpr long long kOneBlock = kOneBlockThreads * kStep;
 
 template <int D>
-__global__ void __launch_bounds__(kOneBlockThreads) k_flag_small(const __grid_constant__ Grid g, int la, bool check)
+__global__ void __launch_bounds__(kOneBlockThreads) k_flag_small(const __grid_constant__ Grid g, int la)
 {
     MRLT_ENTER(g);
-    int c = dev_mark<D>(g, la, g.L - 1, la);
+    dev_mark<D>(g, la, g.L - 1, la);
     for (int l = g.L - 1; l > la; --l) {
         __syncthreads();
-        c += dev_close<D>(g, l);
+        dev_close<D>(g, l);
     }
-    if (check) room_decide(g, c, la);
 }
 
 template <int D, int M, class T>
@@ -394,7 +395,7 @@ static void adapt_dm(Launcher& L, int la, bool check)
     ++L.n;
     if constexpr (D == 1) {
         if (g.N[g.L] <= kOneBlock) {
-            pdl_launch(k_flag_small<D>, 1, kOneBlockThreads, 0, L.st, g, la, check);
+            pdl_launch(k_flag_small<D>, 1, kOneBlockThreads, 0, L.st, g, la);
             ++L.n;
             return;
         }
