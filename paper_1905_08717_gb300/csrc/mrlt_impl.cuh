@@ -812,9 +812,13 @@ struct Launch; // fwd
 // sync: see TreeSync; tick: the index of its tile tickets in g.built.
 int launch_stage(const Grid& g, cudaStream_t st, int lo, int hi, int s, int lmin, double b, int reg, TreeSync sync,
                  int tick);
+// iterations of the longest captured piece and its lead (see run_macro).  Measured
+// on a GB300, whole passes with 8 / 16 / 32: 1D Burgers L = 10 from creation 19.2 /
+// 19.1 / 19.8 ms, mixed 2D Euler opening 78.1 / 78.9 / 80.5, 2D Burgers 83.9 / 83.8 /
+// 85.0, a batch of 24 66.6 / 67.7 / 72.5, a server's 12 requests 55.4 / 56.4 / 58.7.
+constexpr int kBlockIters = 16;
 // words of g.built: three, and one for each stage launch of a captured piece (at
 // most kBlockIters iterations of one launch and two for each level)
-constexpr int kBlockIters = 16;
 constexpr int kDirectTick = 2, kFirstTick = 3;
 constexpr int kBuiltWords = kFirstTick + kBlockIters * (1 + 2 * (LMAX + 1));
 void launch_wave(const Grid& g, cudaStream_t st);

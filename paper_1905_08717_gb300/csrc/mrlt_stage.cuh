@@ -106,7 +106,9 @@ struct TileShape {
     // CTAs per SM that the registers are shared out for.  Measured on a GB300,
     // solves of the benchmark cases: 2D FP32 4 / 5 / 6 per SM 99.3 / 97.1 / 97.4
     // ms, 3D FP32 2 / 3 / 4 24.6 / 22.7 / 22.8 ms; 2D FP64 2 / 3 / 4 / 5 240 /
-    // 221.5 / 221.7 / 222.8 ms, 3D FP64 1 / 2 48.2 / 43.3 ms (bound by FP64 issue).
+    // 221.5 / 221.7 / 222.8 ms, 3D FP64 1 / 2 48.2 / 43.3 ms (bound by FP64 issue);
+    // 1D FP64 4 / 8 / 16: Sod L = 10 18.63 / 18.46 / 19.20 ms, its full grid at L = 14
+    // 4.48 / 4.97 / 5.31 ms, Burgers L = 14 2.84 / 2.84 / 3.01 ms.
     static constexpr int PERSM = D == 1 ? 8 : (D == 2 ? (sizeof(R) == 4 ? 5 : 3) : (sizeof(R) == 4 ? 3 : 2));
 };
 

@@ -82,3 +82,25 @@ def test_direct_launches_equal_replayed_pieces(dim, eq, L, lb, mode, rk):
     assert np.array_equal(va, vb) and np.array_equal(va, vc)
     for s in (a, b, c):
         s.close()
+
+
+@pytest.mark.parametrize("rk,mode", [(3, I.TIME_LT), (2, I.TIME_LT), (2, I.TIME_GTS)])
+def test_macro_step_of_2048_iterations(rk, mode):
+    """eleven levels above the coarsest: 128 leads and blocks per macro step,
+    against the oracle (the same leaves, values to the parity tolerance of the
+    adaptive 1D tests) and against direct launches, bit for bit"""
+    import oracle
+    import paper_1905_08717_gb300 as pkg
+    p, q = I.burgers_1d(L=12, min_level=1, rk_order=rk)
+    p = p.replace(time_mode=mode)
+    dt = 0.25 / (1 << 12)
+    a, b, o = pkg.Solver(p, q), pkg.Solver(p, q), oracle.Oracle(p, q)
+    b.profile(True)
+    for s in (a, b, o):
+        s.iterate(dt, 2048)
+    (ka, va), (kb, vb), (ko, vo) = a.leaves(), b.leaves(), o.leaves()
+    assert np.array_equal(ka, kb) and np.array_equal(va, vb)
+    assert np.array_equal(ka, ko)
+    assert np.abs(va - vo).max() <= 1e-12 * np.abs(vo).max()
+    a.close()
+    b.close()
