@@ -1200,10 +1200,6 @@ mr_status layout_alloc(mr_solver* h, const mr_config* cfg)
 
 } // namespace
 
-extern "C" {
-
-} // extern "C"
-
 namespace {
 
 mr_status create(const mr_config* cfg, const double* q0, bool copy_input, void* cuda_stream, mr_solver** out)

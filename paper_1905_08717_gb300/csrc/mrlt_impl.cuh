@@ -25,7 +25,7 @@
 //       change while its register holds a value (the restricted remesh keeps
 //       both sides until the coarse step ends, when the reflux clears them).
 //   - per-level compact lists (int32) of leaves and internal nodes, ascending
-//     cell id, rebuilt after every remesh by warp-ballot stream compaction.
+//     cell id, rebuilt after every remesh by a two-pass stream compaction.
 //   Free slots form a stack (fstack, ftop[0] entries); a remesh releases the
 //   slots of removed nodes, then pops slots for new nodes (ftop[1] counts the
 //   pops until the next compaction commits them).

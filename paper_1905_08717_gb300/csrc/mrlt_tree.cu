@@ -1,7 +1,7 @@
 // mrlt_tree.cu -- tree kernels of the MRLT library: projections and tree
 // refreshing (Eqs. 3, 15-22; Algs. 3, 4, 6, 8, 9), the multiresolution
 // adaptation (details Eq. 5, thresholding Alg. 2, graded closure Alg. 1),
-// warp-ballot compaction of the per-level leaf / internal-node lists,
+// compaction of the per-level leaf / internal-node / tile lists,
 // conservative flux registers, reductions and read-back packing.
 #include "mrlt_tree.cuh"
 
@@ -30,10 +30,7 @@ static inline int blocks_list(const Grid& g, int l)
 // runs one device body of mrlt_tree_dev.cuh over its own grid; kernels that leave
 // the tree alone look it up before they wait (tree_enter).  Most launches
 // are short chains of dependent trips, so that takes two or three of five trips
-// off them.  Measured on a GB300 with the stage kernel's early start, whole
-// solves: 1D Burgers L = 10 30.5 to 23.6 ms (made from nothing), 2D Burgers
-// L = 10 109.6 to 94.4 ms, 2D Euler L = 10 mixed 67.3 to 59.4 ms, global step
-// L = 9 64.6 to 60.6 ms, 3D blast L = 7 48.4 to 45.6 ms.
+// off them (figures at tree_enter).
 // (T: the storage type of the fields, double or float)
 template <int M, class T>
 __global__ void k_leaf_copy(const __grid_constant__ Grid g, int lo, int hi, int from, int to)
