@@ -1862,6 +1862,14 @@ mr_status batch_fail(mr_batch* b, int i, mr_status r)
 
 extern "C" {
 
+// Batches of this size and more wait before every lookup (TreeSync, kWait).
+// Measured on a GB300, uneven reaction-diffusion problems over the same span,
+// waiting / early: 8 instances 8.6 / 8.1 ms, 24 23.0 / 24.4, 48 43.3 / 46.7, 96 88.0 /
+// 96.3, 160 148 / 164, 256 237 / 266 ms.  From creation, where half of the time is
+// the host's, 24 instances take 71 / 68 ms, hence a line above those.  A server's
+// mix runs alike both ways (60 to 67 requests/s).
+constexpr int kWaitInstances = 32;
+
 mr_status mr_batch_create(int n, const mr_config* cfgs, const double* const* q0s, void* cuda_stream,
                           mr_batch** out, int* failed_index)
 {
@@ -1901,6 +1909,7 @@ mr_status mr_batch_create(int n, const mr_config* cfgs, const double* const* q0s
         // phase (captured graphs), since co-residency of several cooperative
         // grids is not something the instances could rely on
         h->launch_mode = MR_LAUNCH_GRAPH;
+        h->K.wait_first = n >= kWaitInstances;
         b->inst.push_back(h);
     }
     *out = b;

@@ -132,6 +132,9 @@ __device__ __forceinline__ bool halted(const Grid& g) { return g.room[1] != 0; }
 //    taken for that count: word 0, of captured launches, counts within a piece and
 //    is cleared at the end of each (k_piece_end); word 1, of direct launches, only
 //    grows, and the host knows the count.
+//  - kWait: it waits first.  For instances of a large batch, which fill the GPU
+//    for one another: nothing is gained there by starting early, and the acquire
+//    (which drops the L1 cache) slows the neighbours.
 // tree_enter is called by every thread of the CTA and returns whether this one has
 // waited.  Measured on a GB300 against waiting first everywhere: 1D Burgers L = 10
 // 17.9 / 20.9 ms, 2D Burgers L = 10 83.5 / 95.3, global step L = 9 72.0 / 77.1, 3D
@@ -139,7 +142,7 @@ __device__ __forceinline__ bool halted(const Grid& g) { return g.room[1] != 0; }
 // 85.3 ms.  In 2D and 3D one thread reads the count for its CTA (with a read by
 // every warp 2D Burgers took 1% and 2D Euler 1.5% longer); the small CTAs of 1D
 // read it with every thread (one thread and a barrier: 2% longer).
-enum TreeMode { kVisible = 0, kAcquire, kPublish };
+enum TreeMode { kVisible = 0, kAcquire, kPublish, kWait };
 struct TreeSync {
     int mode, word;
     unsigned need;
@@ -154,7 +157,7 @@ __device__ __forceinline__ bool tree_enter(const Grid& g, const TreeSync& t)
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(n) : "l"(g.built + t.word) : "memory");
         const bool there = (int)(n - t.need) >= 0;
         if (D == 1 ? there : __syncthreads_or(there) != 0) return false;
-    } else {
+    } else if (t.mode == kPublish) {
         asm volatile("griddepcontrol.wait;" ::: "memory");
         if (blockIdx.x == 0) { // before this CTA lets the next kernel start
             if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(g.built + t.word) : "memory");

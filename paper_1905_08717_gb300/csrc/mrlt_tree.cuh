@@ -16,10 +16,12 @@ struct Launcher {
     unsigned published[2] = {0, 0}; // publications, of the piece being captured and of direct launches
     bool stale = true;              // something to look up has changed since the last publication
     int stages = 0;                 // stage launches of the piece
+    bool wait_first = false;        // one of many solvers that share the GPU
 
     // how the next kernel that looks the tree up enters
     TreeSync enter()
     {
+        if (wait_first) return {kWait, 0, 0};
         const int word = capturing ? 0 : 1;
         if (!stale) return {capturing && !published[0] ? kVisible : kAcquire, word, published[word]};
         stale = false;

@@ -104,3 +104,20 @@ def test_macro_step_of_2048_iterations(rk, mode):
     assert np.abs(va - vo).max() <= 1e-12 * np.abs(vo).max()
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("n", [31, 32])
+def test_batches_on_both_sides_of_waiting_first(n):
+    """instances of a batch, below the size from which they wait before every
+    lookup and at it, against single solvers, bit for bit"""
+    import paper_1905_08717_gb300 as pkg
+    probs, qs = I.rd_batch(n=n, levels=(6, 8))
+    b = pkg.Batch(probs, qs)
+    b.step(0.004)
+    for i in range(0, n, 5):
+        s = pkg.Solver(probs[i], qs[i])
+        s.step(0.004)
+        for x, y in zip(s.leaves(), b.instances[i].leaves()):
+            assert np.array_equal(x, y), i
+        s.close()
+    b.close()

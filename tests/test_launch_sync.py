@@ -13,6 +13,7 @@ int main(int argc, char** argv)
     for (const char* c = argv[1]; *c; ++c) {
         if (*c == '[') { K.capturing = true; K.stale = false; K.published[0] = 0; K.stages = 0; } // piece_begin
         else if (*c == ']') { K.capturing = false; K.stale = true; }                             // piece_end
+        else if (*c == 'w') K.wait_first = true;
         else if (*c == 'c') K.stale = true; // compaction, resize, fine step, graph launch
         else {
             const TreeSync s = K.enter();
@@ -22,7 +23,7 @@ int main(int argc, char** argv)
     return 0;
 }
 """
-VISIBLE, ACQUIRE, PUBLISH = 0, 1, 2
+VISIBLE, ACQUIRE, PUBLISH, WAIT = range(4)
 
 
 def test_entry_of_launches(tmp_path):
@@ -45,3 +46,5 @@ def test_entry_of_launches(tmp_path):
     got = run("ee[ecee]eece")
     assert got == [(PUBLISH, 1, 1), (ACQUIRE, 1, 1), (VISIBLE, 0, 0), (PUBLISH, 0, 1), (ACQUIRE, 0, 1),
                    (PUBLISH, 1, 2), (ACQUIRE, 1, 2), (PUBLISH, 1, 3)]
+    # a solver that waits first does so everywhere
+    assert {m for m, _, _ in run("we[eece]ece")} == {WAIT}
