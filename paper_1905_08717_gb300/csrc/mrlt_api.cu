@@ -1033,7 +1033,8 @@ bool reads_host_memory()
 // 33 MB 1.04 / 1.11, 84 MB 1.97 / 2.17, 134 MB 3.05 / 3.30, 671 MB 11.3 / 11.8
 // (the release alone takes the same either way); with the host's caches flushed
 // before the call 0.64 / 0.69, 1.17 / 1.24, 2.09 / 2.20, 3.08 / 3.26 and 11.2 /
-// 11.8 ms.  At 8 MB both ways take 0.40 ms.  On a host whose staging was slow a 3D
+// 11.8 ms; beside another thread's solver 1.1 / 2.1, 1.9 / 1.7, 2.2 / 2.3, 3.3 / 3.3 and
+// 11.6 / 12.9 ms.  At 8 MB both ways take 0.40 ms.  On a host whose staging was slow a 3D
 // solve at L = 8 (671 MB, 32 iterations) took 139 ms with the copy and 50 without.
 // A server's own vectors, released right after (h->copy_input), are copied: its
 // mix of 12 requests took 65 ms in place and 60 copied.  The caller's memory is
