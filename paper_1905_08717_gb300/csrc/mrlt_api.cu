@@ -1092,8 +1092,13 @@ mr_status fresh_state(mr_solver* h, const double* q0)
 
 mr_status init_state(mr_solver* h, const double* q0)
 {
+    // g.built starts again at zero: nothing may be told from it (see TreeSync) until
+    // the stream has been waited for, as fresh_state does at its end
+    const bool first = h->K.wait_first;
+    h->K.wait_first = true;
     const mr_status r = fresh_state(h, q0);
     if (r != MR_OK) cudaStreamSynchronize(h->stream); // a kernel may still be reading q0
+    h->K.wait_first = first;
     return r;
 }
 
